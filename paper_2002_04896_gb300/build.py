@@ -1,7 +1,8 @@
 """Build libcroft.so (the C-ABI library) in-tree with nvcc for sm_103a.
 
 Translation units compile in parallel; the pass-kernel instantiations are split
-into four size groups (``croft_kernels.cu`` compiled with ``-DCROFT_GROUP=g``),
+into four size groups (``croft_kernels.cu`` compiled with ``-DCROFT_GROUP=g``), so are
+the two-stage ones (``croft_two.cu``, ``-DCROFT_TWO_GROUP=g``),
 the fused convolution pass into five (``croft_conv.cu``, ``-DCROFT_CONV_GROUP=g``).
 Objects go to ``paper_2002_04896_gb300/_build/`` and are rebuilt only when a
 source or header is newer than the object.
@@ -48,8 +49,11 @@ def _units():
     for g in range(4):
         units.append((os.path.join(CSRC, "croft_tc.cu"), os.path.join(BUILD, f"croft_tc_g{g}.o"),
                       [f"-DCROFT_TC_GROUP={g}"]))
+    for g in range(N_GROUPS):
+        units.append((os.path.join(CSRC, "croft_two.cu"), os.path.join(BUILD, f"croft_two_g{g}.o"),
+                      [f"-DCROFT_TWO_GROUP={g}"]))
     for src in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
-        if os.path.basename(src) in ("croft_kernels.cu", "croft_conv.cu"):
+        if os.path.basename(src) in ("croft_kernels.cu", "croft_conv.cu", "croft_two.cu"):
             continue
         obj = os.path.join(BUILD, os.path.basename(src)[:-3] + ".o")
         units.append((src, obj, []))

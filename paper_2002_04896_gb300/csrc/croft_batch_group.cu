@@ -22,10 +22,16 @@ namespace croft {
 
 typedef void (*group_fn)(const GroupArgs);
 
+template <int LAYOUT, int N>
+static group_fn group_kernel_of() {
+    if constexpr (group_two<LAYOUT, N>().r1 != 0) return croft_group_two_kernel<LAYOUT, N>;
+    else return croft_group_kernel<LAYOUT, N>;
+}
+
 static group_fn group_kernel_for(int layout, int n) {
     switch (n) {
 #define CROFT_G_CASE(N) \
-    case N: return layout == LAYOUT_ROW ? croft_group_kernel<LAYOUT_ROW, N> : croft_group_kernel<LAYOUT_COL, N>;
+    case N: return layout == LAYOUT_ROW ? group_kernel_of<LAYOUT_ROW, N>() : group_kernel_of<LAYOUT_COL, N>();
         CROFT_BATCH_SIZES(CROFT_G_CASE)
 #undef CROFT_G_CASE
         default: return nullptr;
@@ -33,6 +39,7 @@ static group_fn group_kernel_for(int layout, int n) {
 }
 
 int host_build_twiddles(int n, float* out);  // croft_plan.cu
+void host_build_two_twiddles(int n, int r1, float* out);
 
 struct GroupLaunch {
     int pass, layout, n;
@@ -71,7 +78,7 @@ croft_status group_state_build(const std::vector<int>& dims, const std::vector<i
     std::vector<GroupSeg> segs;
     std::vector<unsigned short> cta;
     std::vector<float> pool;
-    std::map<int, int> tw_off;
+    std::map<std::pair<int, int>, int> tw_off;  // (length, first radix of a two-stage pass or 0) -> offset
     // first pass of each grid (lowest pass index whose axis is longer than 1)
     std::vector<int> first(pgrid.size(), -1);
     for (size_t i = 0; i < pgrid.size(); ++i)
@@ -94,26 +101,37 @@ croft_status group_state_build(const std::vector<int>& dims, const std::vector<i
                 group_state_destroy(s);
                 return CROFT_ERR_UNSUPPORTED_SIZE;
             }
-            if (!tw_off.count(n)) {
-                tw_off[n] = (int)(pool.size() / 2);
+            const bool row = layout == LAYOUT_ROW;
+            const CroftTwo K = row ? croft_two_row(n) : croft_two_col(n, false);
+            const std::pair<int, int> key{n, K.r1};
+            if (!tw_off.count(key)) {
+                tw_off[key] = (int)(pool.size() / 2);
                 std::vector<float> t(2 * (size_t)n + 2, 0.f);
-                if (n > 1 && host_build_twiddles(n, t.data()) != n - 1) {
+                if (K.r1) {
+                    host_build_two_twiddles(n, K.r1, t.data());
+                } else if (n > 1 && host_build_twiddles(n, t.data()) != n - 1) {
                     group_state_destroy(s);
                     return CROFT_ERR_UNSUPPORTED_SIZE;
                 }
-                pool.insert(pool.end(), t.begin(), t.begin() + 2 * std::max(1, n - 1));
+                pool.insert(pool.end(), t.begin(), t.begin() + 2 * n);
             }
-            const int T = croft_threads_per_pencil(n);
-            const int tw_pad = ((n + 1) / 2) * 2;
             GroupLaunch L;
             L.pass = p;
             L.layout = layout;
             L.n = n;
-            L.W = layout == LAYOUT_ROW ? 256 / T : croft_col_width(n, 8);
-            L.block = L.W * T;
-            const long long tile_elems = layout == LAYOUT_ROW ? (long long)L.W * croft_row_ld_staged(n) : (long long)n * L.W;
-            L.smem = (int)((tw_pad + tile_elems) * sizeof(float2));
-            L.tw_off = tw_off[n];
+            if (K.r1) {
+                L.W = K.w;
+                L.block = K.w * K.t;
+                L.smem = croft_two_smem(K, n, row);
+            } else {
+                const int T = croft_threads_per_pencil(n);
+                const int tw_pad = ((n + 1) / 2) * 2;
+                L.W = row ? 256 / T : croft_col_width(n, 8);
+                L.block = L.W * T;
+                const long long tile_elems = row ? (long long)L.W * croft_row_ld_staged(n) : (long long)n * L.W;
+                L.smem = (int)((tw_pad + tile_elems) * sizeof(float2));
+            }
+            L.tw_off = tw_off[key];
             L.seg_begin = (int)segs.size();
             L.cta_begin = (int)cta.size();
             for (int i : kv.second) {

@@ -9,9 +9,14 @@
 // Radix 8, 9, 15 and 16 are split Cooley-Tukey (2x4, 3x3, 5x3 and 4x4) with the
 // inner twiddles as compile-time constants; 3 and 5 use the symmetric cos/sin form.  The
 // constants are the exact mathematical values rounded to the working precision
-// (float for complex64, double for complex128).
+// (float for complex64, double for complex128).  The larger radices of the two-stage
+// passes (6, 10, 12, 18 .. 32: DftSplit) take the same split with the inner twiddles
+// computed at compile time.
 #pragma once
 #include <cuda_runtime.h>
+
+#include <type_traits>
+#include <utility>
 
 namespace croft {
 
@@ -245,5 +250,96 @@ template <class C> struct Dft<15, C> {
 };
 
 template <int R, class C> __device__ __forceinline__ void dft(C* v) { Dft<R, C>::run(v); }
+
+// ---------------------------------------------------------------------------
+// composite radices with compile-time inner twiddles
+// ---------------------------------------------------------------------------
+
+// cos(2 pi m / R) in float64 at compile time: the angle is folded into the first octant by
+// integer arithmetic (exact), where 14 Taylor terms leave an error far below half a ulp.
+constexpr double kPi = 3.14159265358979323846264338327950288;
+constexpr double octant_sin(double x) {
+    double t = x, s = x;
+    for (int i = 1; i < 14; ++i) {
+        t *= -x * x / ((2 * i) * (2 * i + 1));
+        s += t;
+    }
+    return s;
+}
+constexpr double octant_cos(double x) {
+    double t = 1, s = 1;
+    for (int i = 1; i < 14; ++i) {
+        t *= -x * x / ((2 * i - 1) * (2 * i));
+        s += t;
+    }
+    return s;
+}
+constexpr double cos_2pi(long long m, long long R) {
+    m = ((m % R) + R) % R;
+    if (2 * m > R) m = R - m;
+    if (4 * m > R) return -cos_2pi(R - 2 * m, 2 * R);
+    if (8 * m <= R) return octant_cos(2 * kPi * (double)m / (double)R);
+    return octant_sin(2 * kPi * (double)(R - 4 * m) / (double)(4 * R));
+}
+constexpr double sin_2pi(long long m, long long R) { return cos_2pi(4 * m - R, 4 * R); }
+
+// f(integral_constant<int, 0>) ... f(integral_constant<int, N - 1>): a loop whose index is a constant
+// expression, so that every twiddle is computed by the compiler.
+template <class F, int... I>
+__device__ __forceinline__ void for_each_index(F&& f, std::integer_sequence<int, I...>) {
+    (f(std::integral_constant<int, I>{}), ...);
+}
+template <int N, class F> __device__ __forceinline__ void for_each_index(F&& f) {
+    for_each_index(f, std::make_integer_sequence<int, N>{});
+}
+
+// a * exp(-2 pi i M / R)
+template <int R, int M, class C> __device__ __forceinline__ C mul_root(C a) {
+    using T = typename CxScalar<C>::T;
+    constexpr int m = ((M % R) + R) % R;
+    if constexpr (m == 0) return a;
+    else if constexpr (4 * m == R) return mul_mi(a);
+    else if constexpr (2 * m == R) return mkc<C>(-a.x, -a.y);
+    else if constexpr (4 * m == 3 * R) return mkc<C>(-a.y, a.x);
+    else {
+        constexpr double c = cos_2pi(m, R), s = -sin_2pi(m, R);
+        return mul_cs(a, (T)c, (T)s);
+    }
+}
+
+// Radix R = A * B: j = B*j1 + j2; length-A DFTs over j1, twiddle W_R^(j2*k1), length-B DFTs over
+// j2; output k1 + A*k2.
+template <int A, int B, class C> struct DftSplit {
+    __device__ __forceinline__ static void run(C* v) {
+        C a[A][B];  // a[k1][j2]
+        for_each_index<B>([&](auto j2c) {
+            constexpr int j2 = decltype(j2c)::value;
+            C t[A];
+#pragma unroll
+            for (int j1 = 0; j1 < A; ++j1) t[j1] = v[B * j1 + j2];
+            Dft<A, C>::run(t);
+            for_each_index<A>([&](auto k1c) {
+                constexpr int k1 = decltype(k1c)::value;
+                a[k1][j2] = mul_root<A * B, j2 * k1>(t[k1]);
+            });
+        });
+#pragma unroll
+        for (int k1 = 0; k1 < A; ++k1) {
+            Dft<B, C>::run(a[k1]);
+#pragma unroll
+            for (int k2 = 0; k2 < B; ++k2) v[k1 + A * k2] = a[k1][k2];
+        }
+    }
+};
+template <class C> struct Dft<6, C> : DftSplit<3, 2, C> {};
+template <class C> struct Dft<10, C> : DftSplit<5, 2, C> {};
+template <class C> struct Dft<12, C> : DftSplit<4, 3, C> {};
+template <class C> struct Dft<18, C> : DftSplit<9, 2, C> {};
+template <class C> struct Dft<20, C> : DftSplit<5, 4, C> {};
+template <class C> struct Dft<24, C> : DftSplit<8, 3, C> {};
+template <class C> struct Dft<25, C> : DftSplit<5, 5, C> {};
+template <class C> struct Dft<27, C> : DftSplit<9, 3, C> {};
+template <class C> struct Dft<30, C> : DftSplit<15, 2, C> {};
+template <class C> struct Dft<32, C> : DftSplit<8, 4, C> {};
 
 }  // namespace croft

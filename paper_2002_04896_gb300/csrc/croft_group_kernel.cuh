@@ -11,6 +11,7 @@
 #pragma once
 #include "croft_fft_core.cuh"
 #include "croft_internal.h"
+#include "croft_two_stage_kernel.cuh"
 
 namespace croft {
 
@@ -26,13 +27,58 @@ struct GroupSeg {
 struct GroupArgs {
     const GroupSeg* segs;           // this launch's segments (device table, pointers filled per exec)
     const unsigned short* cta_seg;  // segment of each CTA
-    const float2* tw;               // twiddle table of N (N-1 entries)
-    int W;                          // ROW: pencils per CTA
+    const float2* tw;               // twiddle table of N (two-stage: N entries; else N-1)
+    int W;                          // ROW, not two-stage: pencils per CTA
     float isign;                    // +1 forward, -1 backward
 };
 
-// ROW launches: W = 256 / T pencils per CTA; COL launches: the compile-time width
-// croft_col_width(N).
+// Batch row and column of pencil `col` of a COL segment.
+__device__ __forceinline__ long long group_col_base(const GroupSeg& S, long long col, int n) {
+    long long b, m;
+    if (S.cdiv.m) {
+        const unsigned q = croft_coldiv_q(S.cdiv.m, S.cdiv.s1, S.cdiv.s2, (unsigned)col);
+        b = q;
+        m = (unsigned)col - q * (unsigned)S.M;
+    } else {
+        b = col / S.M;
+        m = col - b * S.M;
+    }
+    return b * (long long)n * S.M + m;
+}
+
+// The two-stage passes (croft_two_stage_kernel.cuh) of the lengths that have them: the same tiles
+// and arithmetic as a single grid's passes.
+template <int LAYOUT, int N>
+constexpr CroftTwo group_two() { return LAYOUT == LAYOUT_ROW ? croft_two_row(N) : croft_two_col(N, false); }
+
+template <int LAYOUT, int N>
+__global__ void __launch_bounds__(group_two<LAYOUT, N>().w* group_two<LAYOUT, N>().t, group_two<LAYOUT, N>().minb)
+    croft_group_two_kernel(const __grid_constant__ GroupArgs A) {
+    constexpr CroftTwo K = group_two<LAYOUT, N>();
+    extern __shared__ __align__(16) float2 two_smem[];
+    float2* buf = two_smem + (K.stage ? croft_two_pad(N) : 0);
+    pdl_allow_dependents();
+    const float2* tw = two_twiddles<N, K.stage != 0>(A.tw, two_smem, K.w * K.t);
+    const GroupSeg S = A.segs[A.cta_seg[blockIdx.x]];
+    const long long tile = (long long)blockIdx.x - S.first_tile;
+    pdl_wait();
+    if constexpr (LAYOUT == LAYOUT_ROW) {
+        const int c = threadIdx.x / K.t, lane = threadIdx.x % K.t;
+        const long long col = tile * K.w + c;
+        const long long base = col * N;
+        two_pencil<N, K.r1, K.t>(GlobalInUnit{S.in + base, A.isign}, GlobalOutUnit{S.out + base, A.isign},
+                                 TwoExRow<K.r1, float2>{buf + c * K.ld}, tw, lane, col < S.ncols);
+    } else {
+        const int c = threadIdx.x % K.w, lane = threadIdx.x / K.w;
+        const long long col = tile * K.w + c;
+        const long long base = group_col_base(S, col, N);
+        two_pencil<N, K.r1, K.t>(GlobalIn{S.in + base, S.M, A.isign}, GlobalOut{S.out + base, S.M, A.isign},
+                                 TwoExCol<K.r1, K.w, float2>{buf + c}, tw, lane, col < S.ncols);
+    }
+}
+
+// The other lengths (one stage, or no two-stage kernel).  ROW launches: W = 256 / T pencils per
+// CTA; COL launches: the compile-time width croft_col_width(N).
 template <int LAYOUT, int N>
 __global__ void __launch_bounds__(256) croft_group_kernel(const __grid_constant__ GroupArgs A) {
     constexpr int T = croft_threads_per_pencil(N);
@@ -62,16 +108,7 @@ __global__ void __launch_bounds__(256) croft_group_kernel(const __grid_constant_
         const int lane = threadIdx.x / WC;
         const long long col = tile * WC + c;
         const bool ok = col < S.ncols;
-        long long b, m;
-        if (S.cdiv.m) {
-            const unsigned q = croft_coldiv_q(S.cdiv.m, S.cdiv.s1, S.cdiv.s2, (unsigned)col);
-            b = q;
-            m = (unsigned)col - q * (unsigned)S.M;
-        } else {
-            b = col / S.M;
-            m = col - b * S.M;
-        }
-        const long long base = b * (long long)N * S.M + m;
+        const long long base = group_col_base(S, col, N);
         fft_pencil<N, T>(GlobalIn{S.in + base, S.M, A.isign}, SmemColFixed<float2, WC>{sbuf + c},
                          GlobalOut{S.out + base, S.M, A.isign}, stw, lane, ok);
     }

@@ -86,6 +86,14 @@ struct PlaneKernel {
 
 enum PassKind { PASS_AXIS = 0, PASS_PLANE = 1 };
 
+// The two-stage kernel that runs an axis pass in place of its three-stage one (croft_two_stage.h).
+struct TwoLaunch {
+    pass_fn fn;        // NULL: the pass runs its other kernel
+    const float2* tw;  // w_n^{jk} at [j * r1 + k]
+    CroftColDiv cdiv;  // for this tile width
+    int r1, T, W, grid, block, smem;
+};
+
 struct PassLaunch {
     int kind;           // PASS_AXIS or PASS_PLANE
     long long offset;   // element offset of this launch's sub-grid (slab schedule), 0 otherwise
@@ -99,6 +107,7 @@ struct PassLaunch {
     int f64;            // 1: complex128 pass kernel
     int sv;             // schedule variant of a plain pass kernel (croft_pass_sched_v)
     int th;             // threads per pencil of a plain COL pass kernel if not the rule's (0: the rule's)
+    TwoLaunch two;      // two-stage kernel of this pass (croft_two_stage_kernel.cuh)
     int pair;           // 1: cluster-pair column kernel (croft_pair_kernel.cuh)
     int ring;           // 1: tensor-copy ring kernel (RingArgs below)
     RingArgs ra;
@@ -127,6 +136,14 @@ pass_fn lookup_pass_kernel_group_0(int layout, int n, int w, int sv, int th);
 pass_fn lookup_pass_kernel_group_1(int layout, int n, int w, int sv, int th);
 pass_fn lookup_pass_kernel_group_2(int layout, int n, int w, int sv, int th);
 pass_fn lookup_pass_kernel_group_3(int layout, int n, int w, int sv, int th);
+
+// croft_two.cu, one per size group: the two-stage pass kernels (NULL when the length has none)
+pass_fn lookup_two_kernel_group_0(int layout, int n, bool long_stride);
+pass_fn lookup_two_kernel_group_1(int layout, int n, bool long_stride);
+pass_fn lookup_two_kernel_group_2(int layout, int n, bool long_stride);
+pass_fn lookup_two_kernel_group_3(int layout, int n, bool long_stride);
+// Shape of the two-stage kernel of a complex64 pass; two.fn stays NULL when there is none for it.
+void shape_two(TwoLaunch& two, int layout, int n, long long M, long long ncols);
 
 // croft_tc.cu: tensor-core pass kernels (NULL when n has no instantiation); prec 0 = split
 // bf16, 1 = split fp16 with per-butterfly power-of-two scaling (TcPrec)

@@ -6,6 +6,7 @@
 #include <mutex>
 
 #include "croft_internal.h"
+#include "croft_two_stage.h"
 
 namespace croft {
 
@@ -217,6 +218,33 @@ conv_fn conv_kernel_for(int n) {
     return f;
 }
 
+void shape_two(TwoLaunch& two, int layout, int n, long long M, long long ncols) {
+    memset(&two, 0, sizeof(two));
+    const bool row = layout == LAYOUT_ROW, lng = !row && M * (long long)sizeof(float2) > kTwoLongStride;
+    const CroftTwo K = row ? croft_two_row(n) : croft_two_col(n, lng);
+    if (K.r1 == 0) return;
+    pass_fn f = lookup_two_kernel_group_0(layout, n, lng);
+    if (!f) f = lookup_two_kernel_group_1(layout, n, lng);
+    if (!f) f = lookup_two_kernel_group_2(layout, n, lng);
+    if (!f) f = lookup_two_kernel_group_3(layout, n, lng);
+    if (!f) return;
+    const int smem = croft_two_smem(K, n, row);
+    const long long grid = (ncols + K.w - 1) / K.w;
+    if (smem > g_max_smem || grid > 0x7fffffffLL) return;
+    if (smem > 48 * 1024 && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    two.fn = f;
+    two.r1 = K.r1;
+    two.T = K.t;
+    two.W = K.w;
+    two.grid = (int)grid;
+    two.block = K.w * K.t;
+    two.smem = smem;
+    if (!row) two.cdiv = croft_coldiv_make(M, ncols + K.w);
+}
+
 // attr must have room for two entries: the cluster shape and, with pdl, programmatic serialisation.
 static cudaLaunchConfig_t plane_config(const PassLaunch& L, cudaStream_t s, cudaLaunchAttribute* attr, bool pdl = false) {
     cudaLaunchConfig_t cfg = {};
@@ -239,9 +267,10 @@ static cudaLaunchConfig_t plane_config(const PassLaunch& L, cudaStream_t s, cuda
 }
 
 // Plain launch of a pass-shaped kernel, with programmatic stream serialisation when pdl
-// (the kernel must call pdl_wait() before reading what the previous launch wrote).
-template <class... P, class... A>
-static cudaError_t launch_ex(void (*f)(P...), const PassLaunch& L, cudaStream_t s, bool pdl, A... args) {
+// (the kernel must call pdl_wait() before reading what the previous launch wrote).  Shape: a
+// PassLaunch or TwoLaunch.
+template <class Shape, class... P, class... A>
+static cudaError_t launch_ex(void (*f)(P...), const Shape& L, cudaStream_t s, bool pdl, A... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)L.grid, 1, 1);
     cfg.blockDim = dim3((unsigned)L.block, 1, 1);
@@ -307,6 +336,13 @@ cudaError_t launch_pass(const PassLaunch& L, const void* vin, void* vout, cudaSt
         cudaLaunchAttribute attr[2];
         cudaLaunchConfig_t cfg = plane_config(L, s, attr, pdl);
         return cudaLaunchKernelEx(&cfg, L.pk.fn, in, out, L.pargs);
+    }
+    if (L.two.fn) {
+        PassArgs a = L.args;
+        a.tw = L.two.tw;
+        a.W = L.two.W;
+        a.cdiv = L.two.cdiv;
+        return launch_ex(L.two.fn, L.two, s, pdl, in, out, a);
     }
     if (L.pair) {
         pass_fn f = pair_kernel_for(L.args.n);

@@ -100,6 +100,16 @@ static int build_twiddles(int n, const int* radices, int ns, float* out) {
 }
 
 namespace croft {
+// Twiddles of a two-stage pass n = r1 * r2: w_n^{jk} at [j * r1 + k], j < r2, k < r1 (n entries).
+void host_build_two_twiddles(int n, int r1, float* out) {
+    for (int j = 0; j < n / r1; ++j)
+        for (int k = 0; k < r1; ++k) {
+            double re, im;
+            twiddle64((long long)j * k, n, &re, &im);
+            out[2 * (j * r1 + k)] = (float)re;
+            out[2 * (j * r1 + k) + 1] = (float)im;
+        }
+}
 // twiddle table of a length-n axis in the library's schedule (n-1 entries); used by batched plans
 int host_build_twiddles(int n, float* out) {
     int rad[CROFT_MAX_STAGES];
@@ -192,6 +202,27 @@ static int rules_sv(croft_plan p, int axis) {
     return croft_col_sv_default(n, 8, M * 8);
 }
 
+// Gives pass L over the axis its two-stage kernel where the length has one (croft_two_stage.h): the
+// complex64 CUDA-core passes that the rules plan.  A tuned plan's choice and the measurement switches
+// CROFT_RING, CROFT_PAIR and CROFT_COL_TH name a kernel and keep it; CROFT_TWO_STAGE=0 switches the
+// two-stage kernels off.
+static croft_status attach_two(croft_plan p, int axis, PassLaunch& L) {
+    memset(&L.two, 0, sizeof(L.two));
+    const char* te = getenv("CROFT_TWO_STAGE");
+    if (L.f64 || L.tc || p->axis_kind[axis] >= 0 || (te && te[0] == '0') || getenv("CROFT_RING") || getenv("CROFT_PAIR") ||
+        getenv("CROFT_COL_TH"))
+        return CROFT_OK;
+    shape_two(L.two, L.layout, L.args.n, L.args.M, L.args.ncols);
+    if (!L.two.fn) return CROFT_OK;
+    const int n = L.args.n;
+    L.two.tw = p->tw_dev[axis] + n;  // (the axis's second table)
+    std::vector<float> tw(2 * (size_t)n);
+    host_build_two_twiddles(n, L.two.r1, tw.data());
+    return cudaMemcpy((void*)L.two.tw, tw.data(), sizeof(float2) * (size_t)n, cudaMemcpyHostToDevice) == cudaSuccess
+               ? CROFT_OK
+               : CROFT_ERR_CUDA;
+}
+
 static croft_status add_axis_pass(croft_plan p, int axis, int x0 = 0, int nxs = -1, int group = -1, int src_in = -1) {
     const int nx = nxs < 0 ? p->dims[0] : nxs, ny = p->dims[1], nz = p->dims[2];
     const long long N = (long long)nx * ny * nz;
@@ -238,6 +269,8 @@ static croft_status add_axis_pass(croft_plan p, int axis, int x0 = 0, int nxs = 
             L.src_in = sin;
             L.group = grp;
             if (prepare_pass(L) == cudaSuccess) {
+                const croft_status st = attach_two(p, axis, L);
+                if (st != CROFT_OK) return st;
                 p->passes.push_back(L);
                 p->pass_axis.push_back(axis);
                 if (grp >= p->ngroups) p->ngroups = grp + 1;
@@ -297,6 +330,8 @@ static croft_status add_axis_pass(croft_plan p, int axis, int x0 = 0, int nxs = 
     L.src_in = sin;
     L.group = grp;
     if (prepare_pass(L) != cudaSuccess) return CROFT_ERR_CUDA;
+    const croft_status ts = attach_two(p, axis, L);
+    if (ts != CROFT_OK) return ts;
     p->passes.push_back(L);
     p->pass_axis.push_back(axis);
     if (grp >= p->ngroups) p->ngroups = grp + 1;
@@ -527,7 +562,8 @@ static croft_status create_impl(croft_plan* out, int nx, int ny, int nz, croft_d
         }
         std::vector<float> tw(2 * (size_t)(n - 1) + 2, 0.f);
         if (build_twiddles(n, rad, ns, tw.data()) != n - 1) return fail(p, CROFT_ERR_UNSUPPORTED_SIZE);
-        if (dev_alloc((void**)&p->tw_dev[axis], sizeof(float2) * (size_t)n) != cudaSuccess) return fail(p, CROFT_ERR_OOM);
+        // (room for the two-stage passes' table behind it: attach_two)
+        if (dev_alloc((void**)&p->tw_dev[axis], sizeof(float2) * 2 * (size_t)n) != cudaSuccess) return fail(p, CROFT_ERR_OOM);
         if (cudaMemcpy(p->tw_dev[axis], tw.data(), sizeof(float2) * (size_t)(n - 1), cudaMemcpyHostToDevice) != cudaSuccess)
             return fail(p, CROFT_ERR_CUDA);
     }
@@ -617,7 +653,8 @@ static std::string plan_tune_key(int nx, int ny, int nz, croft_dtype dtype) {
     cudaDeviceProp prop;
     cudaGetDeviceProperties(&prop, dev);
     char buf[512];
-    snprintf(buf, sizeof(buf), "plan-v2:%dx%dx%d:%d:%s:%d", nx, ny, nz, (int)dtype, prop.name, rt);
+    // (":two-stage": the rules' kernels that the candidates were timed against)
+    snprintf(buf, sizeof(buf), "plan-v2:%dx%dx%d:%d:%s:%d:two-stage", nx, ny, nz, (int)dtype, prop.name, rt);
     for (char* c = buf; *c; ++c)
         if (*c == ' ' || *c == '"') *c = '_';
     return buf;
@@ -865,6 +902,11 @@ int croft_plan_describe(croft_plan plan, char* buf, int cap) {
         }
         snprintf(tmp, sizeof(tmp), " T=%d W=%d block=%d grid=%d smem=%d", L.T, L.args.W, L.block, L.grid, L.smem);
         s += tmp;
+        if (L.two.fn) {  // the kernel that runs in its place
+            snprintf(tmp, sizeof(tmp), " -> two-stage %dx%d T=%d W=%d block=%d grid=%d smem=%d", L.two.r1, L.args.n / L.two.r1,
+                     L.two.T, L.two.W, L.two.block, L.two.grid, L.two.smem);
+            s += tmp;
+        }
     }
     if (plan->conv_fused) {
         const PassLaunch& L = plan->conv;

@@ -1,0 +1,56 @@
+"""The two-stage passes (needs a GPU): every length that has one, as row pass and as column pass over
+short and long strides with ragged last tiles, against the oracle's axis DFT."""
+
+import math
+
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+LENGTHS = [n for n in (2 ** a * 3 ** b * 5 ** c for a in range(11) for b in range(7) for c in range(5))
+           if 32 < n <= 1024]
+
+
+def _run(croft, shape, axis, direction, seed):
+    rng = np.random.default_rng(seed)
+    x = (rng.uniform(-1, 1, shape) + 1j * rng.uniform(-1, 1, shape)).astype(np.complex64)
+    d = torch.from_numpy(x).cuda()
+    out = torch.full_like(d, complex(float("nan"), 0))
+    with croft.Plan(*shape) as p:
+        desc = p.describe()
+        croft.croft_exec_axes(p.handle, d, out, 1 << axis, direction)
+        croft.croft_exec_axes(p.handle, d, d, 1 << axis, direction)  # in place
+        torch.cuda.synchronize()
+    y = out.cpu().numpy()
+    assert np.array_equal(y.view(np.uint32), d.cpu().numpy().view(np.uint32))
+    return x, y, [s for s in desc.split(" | ") if s.startswith("xyz"[axis] + ":")][0]
+
+
+def _check(x, y, axis, direction):
+    ref = oracle.dft_along_axis(x.astype(np.complex128), axis, direction)
+    e = oracle.rel_l2(y, ref)
+    assert e <= 2e-6 * math.log2(x.shape[axis]), (x.shape, axis, e)  # the bar of a transform of this length
+
+
+@pytest.mark.parametrize("n", sorted(LENGTHS))
+def test_every_length(croft_lib, n):
+    # x: 75 columns; y: 27 columns in each of 2 planes; z: 15 rows (all ragged against the tiles)
+    for shape, axis, direction in (((n, 3, 25), 0, -1), ((2, n, 27), 1, 1), ((5, 3, n), 2, -1)):
+        x, y, desc = _run(croft_lib, shape, axis, direction, n + axis)
+        if n not in (128, 256, 972, 1000):
+            assert "two-stage" in desc, desc
+        _check(x, y, axis, direction)
+
+
+@pytest.mark.parametrize("n", [640, 729, 810, 1024])
+def test_long_strides(croft_lib, n):
+    # elements 262,440 bytes apart: the 16-column tile; 32,805 columns, five in the last tile
+    x, y, desc = _run(croft_lib, (n, 81, 405), 0, -1, n)
+    assert " W=16 " in desc.split("two-stage")[1], desc
+    x, y = x.reshape(n, -1), y.reshape(n, -1)
+    pick = np.r_[0:20, 16380:16390, x.shape[1] - 20:x.shape[1]]
+    _check(x[:, pick], y[:, pick], 0, -1)

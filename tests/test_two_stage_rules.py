@@ -1,0 +1,57 @@
+"""Host checks of the two-stage pass table (``csrc/croft_two_stage.h``): every entry factorises its
+length into radices that have a butterfly, and its tile fits the launch and shared-memory limits it
+names (CPU only)."""
+
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2002_04896_gb300", "csrc")
+RADICES = {2, 3, 4, 5, 6, 8, 9, 10, 12, 15, 16, 18, 20, 24, 25, 27, 30, 32}
+
+PROGRAM = r"""
+#include <cstdio>
+#include "croft_two_stage.h"
+static void put(char k, int n, const CroftTwo& t, bool row) {
+    if (t.r1) std::printf("%c %d %d %d %d %d %d %d %d\n", k, n, t.r1, t.t, t.w, t.minb, t.stage, t.ld, croft_two_smem(t, n, row));
+}
+int main() {
+    for (int n = 1; n <= 5000; ++n) {
+        put('s', n, croft_two_col(n, false), false);
+        put('l', n, croft_two_col(n, true), false);
+        put('r', n, croft_two_row(n), true);
+    }
+    return 0;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def table(tmp_path_factory):
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if not cxx:
+        pytest.skip("no host C++ compiler")
+    d = tmp_path_factory.mktemp("two")
+    (d / "t.cpp").write_text(PROGRAM)
+    subprocess.run([cxx, "-std=c++17", "-I", CSRC, str(d / "t.cpp"), "-o", str(d / "t")], check=True)
+    out = subprocess.run([str(d / "t")], check=True, capture_output=True, text=True).stdout
+    return [(a[0], *map(int, a[1:])) for a in (line.split() for line in out.splitlines())]
+
+
+def test_entries_fit(table):
+    assert len(table) > 100
+    for kind, n, r1, t, w, minb, stage, ld, smem in table:
+        r2 = n // r1
+        assert r1 * r2 == n and r1 in RADICES and r2 in RADICES, (kind, n)
+        threads = w * t
+        assert threads * minb <= 2048 and threads <= 1024, (kind, n, threads, minb)
+        # registers of the launch bound hold the points of the larger butterfly
+        assert min(255, 65536 // (threads * minb)) >= 2 * max(r1, r2), (kind, n)
+        assert minb * (smem + 1024) <= 227 * 1024, (kind, n, smem, minb)
+        if kind == "r":
+            assert ld >= r2 * (r1 + (r1 % 2 == 0)) - (r1 % 2 == 0), (n, ld)
+        else:
+            assert w % 8 == 0, (kind, n, w)  # rows of at least 64 bytes
