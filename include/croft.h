@@ -110,8 +110,10 @@ croft_status croft_plan_create(croft_plan* out, int nx, int ny, int nz, croft_dt
  *       y pass reads the z pass's output from the L2 cache and the grid crosses
  *       HBM about twice per transform; then the x pass.  The paper's chunking of
  *       the transposes into K pieces (Sec. 5.1), here sized to the cache.
- *   CROFT_SCHEDULE_AUTO : THREE_PASS (measured faster on GB300 so far); with the
- *       environment variable CROFT_SCHEDULE_AUTO_FUSED=1, PLANE_FUSED where available.
+ *   CROFT_SCHEDULE_AUTO : THREE_PASS, with the z and y axes of complex64 grids with
+ *       small planes run as one pass over the yz-planes (one plane per CTA, in its shared
+ *       memory: steps 1-5 in one launch); with the environment variable
+ *       CROFT_SCHEDULE_AUTO_FUSED=1, PLANE_FUSED where available.
  *   CROFT_SCHEDULE_TUNED : measured at plan creation (the paper tunes its options 1-4 and
  *       the chunk count K by hand, Sec. 5.1): for each column pass of a 270..512-point axis
  *       the kernel (16- or 8-column tile, near-equal or radix-16-first power-of-two split,
@@ -294,8 +296,8 @@ croft_status croft_exec_backward(croft_plan plan, const void* in, void* out, voi
  * Sec. 4.1).  A process holding an x-slab runs the z and y axes, an all-to-all regroups the
  * grid into y-slabs, and each process then runs the x axis.
  *
- *   plan      : a single-grid plan with one pass per axis (CROFT_SCHEDULE_THREE_PASS, which
- *               AUTO gives); the fused-plane and slab schedules give CROFT_ERR_INVALID_ARG.
+ *   plan      : a single-grid plan with one pass per axis (CROFT_SCHEDULE_THREE_PASS and
+ *               AUTO); the fused-plane and slab schedules give CROFT_ERR_INVALID_ARG.
  *   in, out   : device pointers as for croft_exec_forward (in == out allowed).
  *   axes      : bit a set to transform axis a (0 = x, 1 = y, 2 = z); 0 copies in to out.
  *   direction : -1 forward (Eq. 1), +1 backward (Eq. 2, unnormalised).
@@ -380,7 +382,8 @@ croft_status croft_exec_host_pipeline(croft_plan plan, int count, const void* co
  * its three grid buffers). */
 size_t croft_plan_workspace_bytes(croft_plan plan);
 
-/* Number of kernel launches one exec of this plan issues. */
+/* Number of kernel launches one exec of this plan issues (with timing enabled, croft_plan_set_timing,
+ * AUTO plans take one launch per axis). */
 int croft_plan_num_launches(croft_plan plan);
 
 /*
@@ -393,7 +396,9 @@ int croft_plan_describe(croft_plan plan, char* buf, int cap);
 /*
  * Per-pass timing (tracing hook).  When enabled, each exec records a CUDA
  * event on the exec stream before the first pass and after every logical pass
- * (the slab schedule's z+y launches count as one pass).
+ * (the slab schedule's z+y launches count as one pass).  While it is enabled every axis
+ * runs a pass of its own, also where an AUTO plan otherwise runs z and y as one (the same
+ * transform, rounded differently).
  * croft_plan_pass_times waits for the last exec's events and writes the
  * duration in milliseconds of each pass into ms[0 .. min(cap, passes)-1];
  * it returns the number of passes timed, 0 when timing is off or no exec ran,
@@ -416,8 +421,9 @@ croft_status croft_plan_destroy(croft_plan plan);
 /*
  * Host-side planning helpers (no device needed; used by the tests).
  *
- * croft_factorize - the radix schedule the library uses for a length-n axis,
- * in execution order.  Writes up to cap radices and returns how many stages
+ * croft_factorize - the radix schedule of a length-n axis that the library's
+ * general pass kernels use, in execution order (lengths with a two-stage kernel or a plane
+ * pass split differently there: croft_plan_describe).  Writes up to cap radices and returns how many stages
  * there are, or -1 if n is unsupported.
  *
  * croft_twiddle_table - the float32 twiddle table for a length-n axis and

@@ -399,7 +399,9 @@ static croft_status configure(BatchState* b, int mode) {
     }
     for (int g : b->sgrid) {
         croft_plan sp = nullptr;
-        croft_status st = croft_plan_create(&sp, b->dims[3 * g], b->dims[3 * g + 1], b->dims[3 * g + 2], CROFT_C2C_F32);
+        // (a pass per axis, like the grouped launches: the same bits whichever mode is chosen)
+        croft_status st = croft_plan_create_schedule(&sp, b->dims[3 * g], b->dims[3 * g + 1], b->dims[3 * g + 2], CROFT_C2C_F32,
+                                                     CROFT_SCHEDULE_THREE_PASS);
         if (st != CROFT_OK) return st;
         b->subplans.push_back(sp);
     }

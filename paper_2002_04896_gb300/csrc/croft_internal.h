@@ -86,6 +86,24 @@ struct PlaneKernel {
 
 enum PassKind { PASS_AXIS = 0, PASS_PLANE = 1 };
 
+struct PlanePassArgs {
+    const float2* in;
+    float2* out;
+    const float2* tw_z;      // w_nz^{jk} at [j * R1 + k]
+    const float2* tw_y;      // w_ny^{jk} likewise
+    int nz, r1z, pitch, ld;  // z length, its first radix, slots of a run, elements of a row (croft_plane_pass.h)
+    unsigned div_nz;         // ceil(2^32 / nz): i / nz = umulhi(i, div_nz) for the item numbers of a plane
+    float isign;             // +1 forward, -1 backward (conj-in / conj-out)
+};
+typedef void (*plane_pass_fn)(const PlanePassArgs);
+
+// The z+y pass of a single-grid plan (croft_plane_pass_kernel.cuh), run in place of its z and y passes.
+struct PlanePass {
+    plane_pass_fn fn;    // NULL: none
+    PlanePassArgs args;  // (in, out and isign filled per exec)
+    int grid, block, smem;
+};
+
 // The two-stage kernel that runs an axis pass in place of its three-stage one (croft_two_stage.h).
 struct TwoLaunch {
     pass_fn fn;        // NULL: the pass runs its other kernel
@@ -144,6 +162,11 @@ pass_fn lookup_two_kernel_group_2(int layout, int n, bool long_stride);
 pass_fn lookup_two_kernel_group_3(int layout, int n, bool long_stride);
 // Shape of the two-stage kernel of a complex64 pass; two.fn stays NULL when there is none for it.
 void shape_two(TwoLaunch& two, int layout, int n, long long M, long long ncols);
+
+// croft_plane_pass.cu: the z+y pass over planes of ny rows (NULL when there is none for ny)
+plane_pass_fn plane_pass_kernel_for(int ny);
+cudaError_t plane_pass_prepare(int ny, int smem);
+cudaError_t launch_plane_pass(const PlanePass& P, const float2* in, float2* out, float isign, cudaStream_t s, bool pdl);
 
 // croft_tc.cu: tensor-core pass kernels (NULL when n has no instantiation); prec 0 = split
 // bf16, 1 = split fp16 with per-butterfly power-of-two scaling (TcPrec)

@@ -20,6 +20,7 @@
 #include "../../include/croft.h"
 #include "croft_internal.h"
 #include "croft_plan_internal.h"
+#include "croft_plane_pass.h"
 
 using namespace croft;
 
@@ -359,6 +360,47 @@ static croft_status add_slab_passes(croft_plan p, int planes) {
     return CROFT_OK;
 }
 
+// Whether an exec runs the z and y axes as one pass over the planes: not while it times every axis
+// (croft_plan_set_timing), which takes a launch per axis.
+static bool zy_runs(const croft_plan p) { return p->zy.fn && !p->timing; }
+
+// The z+y pass over whole planes (croft_plane_pass_kernel.cuh), beside the z and y passes that
+// croft_exec_axes and per-axis timing run: AUTO plans of complex64 grids whose planes it takes.
+// CROFT_PLANE_PASS=0 switches it off (measurement).
+static croft_status plan_zy(croft_plan p) {
+    const int nx = p->dims[0], ny = p->dims[1], nz = p->dims[2];
+    const char* pe = getenv("CROFT_PLANE_PASS");
+    if ((pe && pe[0] == '0') || p->passes.size() < 2 || p->pass_axis[0] != 2 || p->pass_axis[1] != 1) return CROFT_OK;
+    if (!croft_plane_pass_rule(nx, ny, nz)) return CROFT_OK;
+    PlanePass z;
+    memset(&z, 0, sizeof(z));
+    z.smem = croft_plane_smem(ny, nz);
+    if (z.smem > g_max_smem) return CROFT_OK;
+    if (plane_pass_prepare(ny, z.smem) != cudaSuccess) {
+        cudaGetLastError();
+        return CROFT_OK;
+    }
+    for (int axis = 1; axis <= 2; ++axis) {
+        const int n = p->dims[axis];
+        std::vector<float> tw(2 * (size_t)n);
+        host_build_two_twiddles(n, croft_plane_r1(n), tw.data());
+        if (cudaMemcpy(p->tw_dev[axis] + 2 * n, tw.data(), sizeof(float2) * (size_t)n, cudaMemcpyHostToDevice) != cudaSuccess)
+            return CROFT_ERR_CUDA;
+    }
+    z.args.tw_z = p->tw_dev[2] + 2 * nz;
+    z.args.tw_y = p->tw_dev[1] + 2 * ny;
+    z.args.nz = nz;
+    z.args.r1z = croft_plane_r1(nz);
+    z.args.pitch = croft_plane_pitch(nz);
+    z.args.ld = croft_plane_ld(nz);
+    z.args.div_nz = (unsigned)((0x100000000ull + (unsigned)nz - 1) / (unsigned)nz);
+    z.grid = nx;
+    z.block = croft_plane_threads(nx, ny, nz);
+    z.fn = plane_pass_kernel_for(ny);
+    p->zy = z;
+    return CROFT_OK;
+}
+
 // Fused z+y pass over every yz-plane (croft_plane_kernel.cuh).
 static croft_status add_plane_pass(croft_plan p, const PlaneKernel* pk) {
     PassLaunch L;
@@ -562,8 +604,8 @@ static croft_status create_impl(croft_plan* out, int nx, int ny, int nz, croft_d
         }
         std::vector<float> tw(2 * (size_t)(n - 1) + 2, 0.f);
         if (build_twiddles(n, rad, ns, tw.data()) != n - 1) return fail(p, CROFT_ERR_UNSUPPORTED_SIZE);
-        // (room for the two-stage passes' table behind it: attach_two)
-        if (dev_alloc((void**)&p->tw_dev[axis], sizeof(float2) * 2 * (size_t)n) != cudaSuccess) return fail(p, CROFT_ERR_OOM);
+        // (room for the tables of the two-stage and plane passes behind it: attach_two, plan_zy)
+        if (dev_alloc((void**)&p->tw_dev[axis], sizeof(float2) * 3 * (size_t)n) != cudaSuccess) return fail(p, CROFT_ERR_OOM);
         if (cudaMemcpy(p->tw_dev[axis], tw.data(), sizeof(float2) * (size_t)(n - 1), cudaMemcpyHostToDevice) != cudaSuccess)
             return fail(p, CROFT_ERR_CUDA);
     }
@@ -610,6 +652,10 @@ static croft_status create_impl(croft_plan* out, int nx, int ny, int nz, croft_d
     for (int i = 0; i < naxes; ++i) {
         if (p->dims[axes[i]] == 1) continue;
         croft_status st = add_axis_pass(p, axes[i]);
+        if (st != CROFT_OK) return fail(p, st);
+    }
+    if (sched == CROFT_SCHEDULE_AUTO && !fused && !want_tc && dtype == CROFT_C2C_F32 && p->axis_kind[1] < 0 && p->axis_kind[2] < 0) {
+        const croft_status st = plan_zy(p);
         if (st != CROFT_OK) return fail(p, st);
     }
     plan_conv(p);
@@ -829,12 +875,14 @@ static croft_status create_tuned(croft_plan* out, int nx, int ny, int nz, croft_
         ch.th[axis] = pick.th;
     }
     // the schedule, as whole forward+backward transforms
-    const croft_schedule scheds[3] = {CROFT_SCHEDULE_THREE_PASS, CROFT_SCHEDULE_SLAB_L2, CROFT_SCHEDULE_PLANE_FUSED};
-    static const char* sn[3] = {"three_pass", "slab_l2", "plane_fused"};
+    // (AUTO differs from THREE_PASS where the rules run z and y as one pass over the planes)
+    const croft_schedule scheds[4] = {CROFT_SCHEDULE_THREE_PASS, CROFT_SCHEDULE_SLAB_L2, CROFT_SCHEDULE_PLANE_FUSED,
+                                      CROFT_SCHEDULE_AUTO};
+    static const char* sn[4] = {"three_pass", "slab_l2", "plane_fused", "plane_pass"};
     double best = 1e30;
-    for (int k = 0; k < 3; ++k) {
+    for (int k = 0; k < (croft_plane_pass_rule(nx, ny, nz) ? 4 : 3); ++k) {
         croft_plan p = nullptr;
-        const croft_status st = create_impl(&p, nx, ny, nz, dtype, scheds[k], k == 0 ? &ch : nullptr);
+        const croft_status st = create_impl(&p, nx, ny, nz, dtype, scheds[k], (k == 0 || k == 3) ? &ch : nullptr);
         if (st != CROFT_OK) {
             cudaGetLastError();
             continue;
@@ -854,7 +902,7 @@ static croft_status create_tuned(croft_plan* out, int nx, int ny, int nz, croft_
     dev_free(x);
     dev_free(y);
     cudaGetLastError();
-    if (sched != CROFT_SCHEDULE_THREE_PASS) ch = AxisChoice();  // the other schedules run the rules' kernels
+    if (sched != CROFT_SCHEDULE_THREE_PASS && sched != CROFT_SCHEDULE_AUTO) ch = AxisChoice();  // the other schedules run the rules' kernels
     plan_tune_store(key, sched, ch, info);
     croft_status st = create_impl(out, nx, ny, nz, dtype, (croft_schedule)sched, &ch);
     if (st == CROFT_OK) (*out)->tuned = "tuned: " + info;
@@ -908,6 +956,12 @@ int croft_plan_describe(croft_plan plan, char* buf, int cap) {
             s += tmp;
         }
     }
+    if (plan->zy.fn) {
+        snprintf(tmp, sizeof(tmp), " | z+y in one pass over the planes: %dx%d, %dx%d block=%d grid=%d smem=%d",
+                 croft_plane_r1(plan->dims[2]), plan->dims[2] / croft_plane_r1(plan->dims[2]), croft_plane_r1(plan->dims[1]),
+                 plan->dims[1] / croft_plane_r1(plan->dims[1]), plan->zy.block, plan->zy.grid, plan->zy.smem);
+        s += tmp;
+    }
     if (plan->conv_fused) {
         const PassLaunch& L = plan->conv;
         snprintf(tmp, sizeof(tmp), " | convolve: %s fwd*G*bwd fused W=%d block=%d grid=%d smem=%d", an[plan->conv_axis],
@@ -943,7 +997,7 @@ size_t croft_plan_workspace_bytes(croft_plan plan) {
 int croft_plan_num_launches(croft_plan plan) {
     if (!plan) return -1;
     if (plan->batch) return batch_num_launches(plan);
-    return plan->passes.empty() ? 0 : (int)plan->passes.size();
+    return (int)plan->passes.size() - (zy_runs(plan) ? 1 : 0);
 }
 
 croft_status croft_plan_set_timing(croft_plan plan, int enable) {
@@ -997,6 +1051,15 @@ croft_status croft_plan_last_device_status(croft_plan plan) {
 // the caller's earlier work in the ordinary way.
 static croft_status run_passes(croft_plan plan, size_t i0, size_t i1, const void* in, void* out, cudaStream_t s,
                                float isign, bool force_out, int* evi, bool& started) {
+    if (i0 == 0 && i1 >= 2 && zy_runs(plan)) {  // z and y as one pass
+        const bool pdl = plan->pdl && started;
+        started = true;
+        if (launch_plane_pass(plan->zy, (const float2*)(force_out ? out : in), (float2*)out, isign, s, pdl) != cudaSuccess) {
+            cudaGetLastError();
+            return CROFT_ERR_CUDA;
+        }
+        i0 = 2;
+    }
     for (size_t i = i0; i < i1; ++i) {
         PassLaunch L = plan->passes[i];
         L.args.isign = isign;

@@ -1,0 +1,57 @@
+// croft_plane_pass.h - the z+y pass over whole yz-planes in shared memory
+// (croft_plane_pass_kernel.cuh): which plane shapes it takes and its launch shape.
+#pragma once
+
+#include "croft_sched.h"
+
+// First radix of a plane axis of n points, n = R1 * R2, both at most 16 (125: 25): the z and y
+// transforms of a plane take two stages each.  0: no plane kernel for the length.
+CROFT_HD constexpr int croft_plane_r1(int n) {
+    switch (n) {
+        case 32: return 8;
+        case 36: return 6;
+        case 40: return 8;
+        case 45: return 9;
+        case 48: return 8;
+        case 50: return 10;
+        case 54: return 9;
+        case 60: return 10;
+        case 64: return 8;
+        case 72: return 9;
+        case 75: return 15;
+        case 80: return 10;
+        case 81: return 9;
+        case 90: return 10;
+        case 96: return 12;
+        case 100: return 10;
+        case 108: return 12;
+        case 120: return 12;
+        case 125: return 25;
+        case 128: return 16;
+        default: return 0;
+    }
+}
+// Elements from one run of a z transform's second stage to the next in shared memory (odd: no bank conflicts
+// between neighbouring frequencies), and from one row of the plane to the next (odd likewise).
+CROFT_HD constexpr int croft_plane_pitch(int nz) { return (nz / croft_plane_r1(nz)) | 1; }
+CROFT_HD constexpr int croft_plane_ld(int nz) { return (croft_plane_r1(nz) * croft_plane_pitch(nz)) | 1; }
+// Shared memory: [plane: ny rows of ld][slot of every z frequency: nz 16-bit numbers].
+CROFT_HD constexpr int croft_plane_smem(int ny, int nz) { return ny * croft_plane_ld(nz) * 8 + (nz * 2 + 15) / 16 * 16; }
+
+// Whether a plan runs its z and y axes as one pass over the planes.  Measured in graph replays (no host time),
+// three passes over plane pass + x pass: 32^3 1.71, 36^3 1.15, 48^3 1.10, 54^3 1.10, 64^3 0.92, 80^3 0.93,
+// 96^3 0.94, 100^3 1.14, 108^3 0.89; 300 planes of 48^2 1.41, 54^2 1.48, 60^2 1.40, 64^2 1.25, 80^2 1.08, 90^2
+// 1.20, 96^2 1.13, 100^2 1.05, 108^2 1.00, 120^2 0.96; 4 planes of 64^2 0.92, 16 of 96^2 0.69.  Launched one by
+// one, a transform of up to about 64^3 points takes as long as its launches (9 us for three, 5 for two), so
+// planes of up to 4096 points always take it; larger ones up to 10,000 where there are more planes than SMs.
+CROFT_HD constexpr bool croft_plane_pass_rule(int nx, int ny, int nz) {
+    return croft_plane_r1(ny) != 0 && croft_plane_r1(nz) != 0 &&
+           (ny * nz <= 4096 || (ny * nz <= 10000 && nx > 152));
+}
+// Threads of a plane's CTA: enough for one round of butterflies a stage where an SM holds one plane, fewer (and
+// more planes at a time) where there are many.  64^3: 128 / 256 / 384 / 512 / 1024 threads 0.81 / 0.89 / 0.88 /
+// 0.92 / 0.90 of the three passes' speed, 300 planes of 64^2 1.12 / 1.25 / 1.02 / 1.02 / 0.91, 4096 of 32^2
+// 1.20 / 1.15 / 1.04 / 1.05 / 0.79.
+CROFT_HD constexpr int croft_plane_threads(int nx, int ny, int nz) {
+    return nx <= 152 ? 512 : (nx <= 608 ? 256 : (ny * nz <= 1600 ? 128 : 192));
+}

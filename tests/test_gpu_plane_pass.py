@@ -1,0 +1,73 @@
+"""The z+y pass over whole planes (needs a GPU): every length it takes on either axis, both directions,
+in place, inside a convolution, and where the rule takes it."""
+
+import math
+
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+LENGTHS = [32, 36, 40, 45, 48, 50, 54, 60, 64, 72, 75, 80, 81, 90, 96, 100, 108, 120, 125, 128]
+
+
+def _noise(shape, seed):
+    rng = np.random.default_rng(seed)
+    return (rng.uniform(-1, 1, shape) + 1j * rng.uniform(-1, 1, shape)).astype(np.complex64)
+
+
+def _check(croft, shape):
+    x = _noise(shape, sum(shape))
+    tol = 2e-6 * math.log2(x.size)
+    d = torch.from_numpy(x).cuda()
+    with croft.Plan(*shape) as p:
+        assert "z+y in one pass" in p.describe(), p.describe()
+        assert croft.croft_plan_num_launches(p.handle) == (2 if shape[0] > 1 else 1)
+        out = torch.full_like(d, complex(float("nan"), 0))
+        p.forward(d, out)
+        b = p.backward(d)
+        c = d.clone()
+        p.forward(c, c)
+        torch.cuda.synchronize()
+        assert torch.equal(torch.view_as_real(out), torch.view_as_real(c))
+        croft.croft_plan_set_timing(p.handle, True)  # an axis at a time
+        t = p.forward(d)
+        n = len(croft.croft_plan_pass_times(p.handle))
+        assert n == croft.croft_plan_num_launches(p.handle) == (3 if shape[0] > 1 else 2)
+    ref = oracle.forward(x)
+    assert oracle.rel_l2(out.cpu().numpy(), ref) <= tol, shape
+    assert oracle.rel_l2(t.cpu().numpy(), ref) <= tol, shape
+    assert oracle.rel_l2(b.cpu().numpy(), oracle.backward(x)) <= tol, shape
+
+
+@pytest.mark.parametrize("n", LENGTHS)
+def test_every_length_as_y_and_z(croft_lib, n):
+    _check(croft_lib, (3, n, 32))
+    _check(croft_lib, (2, 32, n))
+    if n <= 64:
+        _check(croft_lib, (1, n, n))
+
+
+@pytest.mark.parametrize("shape", [(160, 100, 100), (180, 75, 128), (180, 128, 75), (160, 72, 125), (625, 48, 40)])
+def test_many_planes(croft_lib, shape):
+    _check(croft_lib, shape)
+
+
+def test_convolution_and_rule(croft_lib):
+    shape = (20, 60, 48)
+    x = _noise(shape, 5)
+    g = np.random.default_rng(6).uniform(0.1, 1, shape).astype(np.float32)
+    with croft_lib.Plan(*shape) as p:
+        assert "z+y in one pass" in p.describe() and "fwd*G*bwd fused" in p.describe()
+        y = p.convolve(torch.from_numpy(x).cuda(), torch.from_numpy(g).cuda())
+        torch.cuda.synchronize()
+    assert oracle.rel_l2(y.cpu().numpy(), oracle.convolve(x, g)) <= 4e-6 * math.log2(x.size)
+    for shape, takes in (((64, 64, 64), True), ((64, 72, 64), False), ((162, 72, 64), True), ((162, 108, 108), False),
+                         ((8, 30, 32), False), ((8, 32, 256), False)):
+        with croft_lib.Plan(*shape) as p:
+            assert ("z+y in one pass" in p.describe()) == takes, shape
+        with croft_lib.Plan(*shape, schedule=croft_lib.CROFT_SCHEDULE_THREE_PASS) as p:
+            assert "z+y in one pass" not in p.describe(), shape
