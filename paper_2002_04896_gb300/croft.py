@@ -119,9 +119,30 @@ def croft_status_string(status: int) -> str:
     return _status_string(int(status)).decode()
 
 
+# A small grid's transform takes a few microseconds, so what a call costs here counts.  The current stream
+# as torch.cuda.current_stream() has it, without the Stream object that call builds (3.1 us of the 12.9
+# that a 32^3 forward transform took from Python): two C calls, where this torch has them.
+def _bind_current_stream():
+    try:
+        import torch
+        get_device, get_stream = torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
+        initialized = torch.cuda.is_initialized
+    except Exception:  # noqa: BLE001
+        return None
+    return lambda: get_stream(get_device()) if initialized() else torch.cuda.current_stream().cuda_stream
+
+
+_current_stream = None
+
+
 def _stream_ptr(stream) -> int:
+    global _current_stream
     if stream is None:
         try:
+            if _current_stream is None:
+                _current_stream = _bind_current_stream()
+            if _current_stream is not None:
+                return _current_stream()
             import torch
             return torch.cuda.current_stream().cuda_stream
         except Exception:  # noqa: BLE001
@@ -131,13 +152,24 @@ def _stream_ptr(stream) -> int:
     return int(stream.cuda_stream)
 
 
+_torch = None
+_ALLOWED = {}  # complex128 argument of _check_layout -> the dtypes it accepts
+
+
+def _load_torch():
+    global _torch
+    import torch
+    _ALLOWED.update({None: (torch.complex64, torch.complex128), True: (torch.complex128,), False: (torch.complex64,)})
+    _torch = torch
+    return torch
+
+
 def _check_layout(x, numel=None, complex128=None) -> None:
     """dtype, contiguity and element count of a tensor argument (no device check)."""
-    import torch
+    torch = _torch or _load_torch()
     if not isinstance(x, torch.Tensor):
         raise TypeError("expected a torch CUDA tensor or an integer device address")
-    allowed = ((torch.complex64, torch.complex128) if complex128 is None
-               else ((torch.complex128,) if complex128 else (torch.complex64,)))
+    allowed = _ALLOWED[complex128]
     if x.dtype not in allowed:
         raise ValueError(f"croft: expected {' or '.join(map(str, allowed))}, got {x.dtype}")
     if not x.is_contiguous():
@@ -156,7 +188,6 @@ def _ptr(x, numel=None, complex128=None) -> int:
         return 0
     if isinstance(x, int):
         return x
-    import torch
     _check_layout(x, numel, complex128)
     if not x.is_cuda:
         raise ValueError("croft: tensors must live on a CUDA device")
@@ -338,7 +369,7 @@ def croft_plan_create_batched(dims, dtype: int = CROFT_C2C_F32, mode=None) -> in
 
 
 def _ptr_array(xs, sizes=None):
-    vals = [_ptr(x, None if sizes is None else sizes[i]) for i, x in enumerate(xs)]
+    vals = [x if isinstance(x, int) else _ptr(x, None if sizes is None else sizes[i]) for i, x in enumerate(xs)]
     return (_P * max(1, len(vals)))(*vals)
 
 
@@ -430,31 +461,28 @@ class BatchPlan:
 
     def __init__(self, dims, dtype: int = CROFT_C2C_F32, mode=None):
         self.dims = [tuple(int(v) for v in d) for d in dims]
+        self._sizes = [d[0] * d[1] * d[2] for d in self.dims]
         self.handle = None
         self.handle = croft_plan_create_batched(self.dims, dtype, mode)
 
-    def _check_lists(self, ins, outs):
+    def _pointers(self, ins, outs):
+        """The device addresses of both lists, checked against the grids."""
         if len(ins) != len(self.dims) or len(outs) != len(self.dims):
             raise ValueError("one input and one output per grid")
-        for d, a, b in zip(self.dims, ins, outs):
-            n = d[0] * d[1] * d[2]
-            _ptr(a, n)
-            _ptr(b, n)
+        return ([_ptr(a, n) for a, n in zip(ins, self._sizes)], [_ptr(b, n) for b, n in zip(outs, self._sizes)])
 
     def forward(self, ins, outs=None, stream=None):
         import torch
         if outs is None:
             outs = [torch.empty(d, dtype=torch.complex64, device=x.device) for d, x in zip(self.dims, ins)]
-        self._check_lists(ins, outs)
-        croft_exec_batched_forward(self.handle, ins, outs, stream)
+        croft_exec_batched_forward(self.handle, *self._pointers(ins, outs), stream)
         return outs
 
     def backward(self, ins, outs=None, stream=None):
         import torch
         if outs is None:
             outs = [torch.empty(d, dtype=torch.complex64, device=x.device) for d, x in zip(self.dims, ins)]
-        self._check_lists(ins, outs)
-        croft_exec_batched_backward(self.handle, ins, outs, stream)
+        croft_exec_batched_backward(self.handle, *self._pointers(ins, outs), stream)
         return outs
 
     def describe(self) -> str:
@@ -483,6 +511,7 @@ class Plan:
 
     def __init__(self, nx: int, ny: int, nz: int, dtype: int = CROFT_C2C_F32, schedule=None):
         self.shape = (int(nx), int(ny), int(nz))
+        self._numel = self.shape[0] * self.shape[1] * self.shape[2]
         self.dtype = dtype
         self.handle = None
         if schedule is None:
@@ -493,26 +522,26 @@ class Plan:
     def _out(self, inp, out):
         f64 = self.dtype == CROFT_C2C_F64
         if out is None:
-            import torch
+            torch = _torch or _load_torch()
             out = torch.empty(self.shape, dtype=torch.complex128 if f64 else torch.complex64, device=inp.device)
-        n = self.shape[0] * self.shape[1] * self.shape[2]
+        n = self._numel
         return _ptr(inp, n, f64), _ptr(out, n, f64), out
 
     def forward(self, inp, out=None, stream=None):
         pi, po, out = self._out(inp, out)
-        croft_exec_forward(self.handle, pi, po, stream)
+        _check(_exec_forward(self.handle, pi, po, _stream_ptr(stream)), "croft_exec_forward")
         return out
 
     def backward(self, inp, out=None, stream=None):
         pi, po, out = self._out(inp, out)
-        croft_exec_backward(self.handle, pi, po, stream)
+        _check(_exec_backward(self.handle, pi, po, _stream_ptr(stream)), "croft_exec_backward")
         return out
 
     def convolve(self, inp, g, out=None, stream=None):
         """B(G * F(inp)) with a real influence function g of the grid's shape (float32, or float64 for complex128)."""
         pi, po, out = self._out(inp, out)
-        n = self.shape[0] * self.shape[1] * self.shape[2]
-        croft_exec_convolve(self.handle, pi, po, _real_ptr(g, n, self.dtype == CROFT_C2C_F64), stream)
+        pg = _real_ptr(g, self._numel, self.dtype == CROFT_C2C_F64)
+        _check(_exec_convolve(self.handle, pi, po, pg, _stream_ptr(stream)), "croft_exec_convolve")
         return out
 
     def describe(self) -> str:
