@@ -2,6 +2,7 @@
 // Compiled five times: -DCROFT_CONV_GROUP=0..3 take the four complex64 size groups
 // of croft_sizes.h; 4 takes the complex128 lengths and the multiply-only kernels.
 #include "croft_conv_kernel.cuh"
+#include "croft_two_conv_kernel.cuh"
 #include "croft_sizes.h"
 
 #ifndef CROFT_CONV_GROUP
@@ -10,8 +11,14 @@
 
 namespace croft {
 
+// The lengths with a two-stage kernel take that one, the others the general one.
+template <int N>
+static conv_fn conv_of() {
+    if constexpr (croft_two_conv(N).r1 != 0) return croft_two_conv_kernel<N>;
+    else return conv_kernel_of<N, float2>();
+}
 #define CROFT_CONV_CASE(N) \
-    case N: return conv_kernel_of<N, float2>();
+    case N: return conv_of<N>();
 
 #define CROFT_CAT_(a, b) a##b
 #define CROFT_CAT(a, b) CROFT_CAT_(a, b)

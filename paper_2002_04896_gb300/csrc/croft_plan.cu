@@ -21,6 +21,7 @@
 #include "croft_internal.h"
 #include "croft_plan_internal.h"
 #include "croft_plane_pass.h"
+#include "croft_two_stage.h"
 
 using namespace croft;
 
@@ -161,7 +162,6 @@ croft_status croft_plan_destroy(croft_plan plan) {
         dev_free(plan->tw_dev[a]);
         dev_free(plan->tw_pair[a]);
     }
-    dev_free(plan->tw_conv);
     for (cudaEvent_t e : plan->ev)
         if (e) cudaEventDestroy(e);
     if (plan->batch) batch_state_destroy(plan->batch);
@@ -441,37 +441,48 @@ static void plan_conv(croft_plan p) {
     const long long N = (long long)p->dims[0] * p->dims[1] * p->dims[2];
     const long long M = (axis == 2) ? 1 : (axis == 1 ? (long long)p->dims[2] : (long long)p->dims[1] * p->dims[2]);
     if (f64 ? !conv64_kernel_for(n) : !conv_kernel_for(n)) return;
-    // the fused kernel runs the column schedule; the axis's twiddle table follows its pass's,
-    // so a pass on another schedule (the rules' or a tuned radix-16-first split) gives the
-    // convolution a table of its own (complex64)
-    const CroftSched sa = croft_pass_sched_v(n, Lp.layout, f64 ? 16 : 8, Lp.sv),
-                     sb = croft_pass_sched(n, LAYOUT_COL, f64 ? 16 : 8);
-    bool same = sa.count == sb.count;
-    for (int i = 0; same && i < sa.count; ++i) same = sa.r[i] == sb.r[i];
-    if (!same && f64) return;
     PassLaunch L;
-    // the kernel's column width is a compile-time constant (croft_conv_width)
-    const int want_w = croft_conv_width(n, f64 ? 16 : 8);
-    if (!shape_pass(L, LAYOUT_COL, n, M, N / n, false, f64, want_w) || L.args.W != want_w) return;
-    const long long es = f64 ? 16 : 8;
-    const long long smem = ((long long)L.args.tw_pad + (long long)n * L.args.W) * es + (long long)n * L.args.W * (es / 2);
-    if (smem > g_max_smem) return;
-    L.smem = (int)smem;
-    L.kind = PASS_AXIS;
-    L.args.tw = p->tw_dev[axis];
-    if (!same) {
-        std::vector<float> tw(2 * (size_t)(n - 1) + 2, 0.f);
-        if (build_twiddles(n, sb.r, sb.count, tw.data()) != n - 1) return;
-        if (!p->tw_conv) {
-            if (dev_alloc((void**)&p->tw_conv, sizeof(float2) * (size_t)n) != cudaSuccess) {
-                p->tw_conv = NULL;
-                return;
-            }
-            if (cudaMemcpy(p->tw_conv, tw.data(), sizeof(float2) * (size_t)(n - 1), cudaMemcpyHostToDevice) != cudaSuccess)
-                return;
+    const CroftTwo K = f64 ? CroftTwo{0, 0, 0, 0, 0, 0} : croft_two_conv(n);
+    if (K.r1) {  // two stages (croft_two_conv_kernel.cuh)
+        memset(&L, 0, sizeof(L));
+        const long long ncols = N / n, grid = (ncols + K.w - 1) / K.w;
+        if (grid > 0x7fffffffLL) return;
+        L.layout = LAYOUT_COL;
+        L.T = K.t;
+        L.args.n = n;
+        L.args.M = M;
+        L.args.ncols = ncols;
+        L.args.W = K.w;
+        L.args.cdiv = croft_coldiv_make(M, ncols + K.w);
+        L.grid = (int)grid;
+        L.block = K.w * K.t;
+        L.smem = croft_two_conv_smem(K, n);
+        if (L.smem > g_max_smem) return;
+        std::vector<float> tw(2 * (size_t)n);
+        host_build_two_twiddles(n, K.r1, tw.data());
+        float2* d = p->tw_dev[axis] + 3 * n;  // (the axis's fourth table)
+        if (cudaMemcpy(d, tw.data(), sizeof(float2) * (size_t)n, cudaMemcpyHostToDevice) != cudaSuccess) {
+            cudaGetLastError();
+            return;
         }
-        L.args.tw = p->tw_conv;
+        L.args.tw = d;
+    } else {
+        // the general kernel runs the column schedule on the axis's own twiddle table
+        const CroftSched sa = croft_pass_sched_v(n, Lp.layout, f64 ? 16 : 8, Lp.sv),
+                         sb = croft_pass_sched(n, LAYOUT_COL, f64 ? 16 : 8);
+        bool same = sa.count == sb.count;
+        for (int i = 0; same && i < sa.count; ++i) same = sa.r[i] == sb.r[i];
+        if (!same) return;
+        // the kernel's column width is a compile-time constant (croft_conv_width)
+        const int want_w = croft_conv_width(n, f64 ? 16 : 8);
+        if (!shape_pass(L, LAYOUT_COL, n, M, N / n, false, f64, want_w) || L.args.W != want_w) return;
+        const long long es = f64 ? 16 : 8;
+        const long long smem = ((long long)L.args.tw_pad + (long long)n * L.args.W) * es + (long long)n * L.args.W * (es / 2);
+        if (smem > g_max_smem) return;
+        L.smem = (int)smem;
+        L.args.tw = p->tw_dev[axis];
     }
+    L.kind = PASS_AXIS;
     L.args.tw64 = f64 ? (const double2*)p->tw_dev[axis] : nullptr;
     L.args.status = p->d_status;
     L.group = Lp.group;
@@ -535,7 +546,6 @@ static croft_status create_impl(croft_plan* out, int nx, int ny, int nz, croft_d
         p->tw_dev[a] = NULL;
         p->tw_pair[a] = NULL;
     }
-    p->tw_conv = NULL;
     p->timing = false;
     p->ev_count = 0;
     p->ngroups = 0;
@@ -604,8 +614,8 @@ static croft_status create_impl(croft_plan* out, int nx, int ny, int nz, croft_d
         }
         std::vector<float> tw(2 * (size_t)(n - 1) + 2, 0.f);
         if (build_twiddles(n, rad, ns, tw.data()) != n - 1) return fail(p, CROFT_ERR_UNSUPPORTED_SIZE);
-        // (room for the tables of the two-stage and plane passes behind it: attach_two, plan_zy)
-        if (dev_alloc((void**)&p->tw_dev[axis], sizeof(float2) * 3 * (size_t)n) != cudaSuccess) return fail(p, CROFT_ERR_OOM);
+        // (room for three more tables behind it: attach_two, plan_zy, plan_conv)
+        if (dev_alloc((void**)&p->tw_dev[axis], sizeof(float2) * 4 * (size_t)n) != cudaSuccess) return fail(p, CROFT_ERR_OOM);
         if (cudaMemcpy(p->tw_dev[axis], tw.data(), sizeof(float2) * (size_t)(n - 1), cudaMemcpyHostToDevice) != cudaSuccess)
             return fail(p, CROFT_ERR_CUDA);
     }

@@ -10,7 +10,10 @@
 //   middle, butterfly k < R1    elements k + j*R1 -> twiddles, radix R2, conj(G * .), radix R2 -> the same slots
 //   backward stage 2, butterfly b < R2   elements b*R1 + j, twiddles w_N^{jb}, radix R1, conj -> y[b + j*R2]
 // (the backward transform is conj o F o conj).  The middle stage works in place, so no barrier
-// stands between its reads and its writes.  Every thread copies the G values of its own middle
+// stands between its reads and its writes.  The three-stage kernel crossed shared memory four times with a barrier
+// on either side of each; this one is bounded by the latency of its three phases at two to four CTAs per
+// SM (data and G tiles) and, at 256 points and below, by instruction issue: 134M points (2.7 GB) at 256
+// points 602 -> 527 us, at 512 points 755 -> 580.  Every thread copies the G values of its own middle
 // butterflies to shared memory (cp.async at entry, behind the forward stage) and reads only those.
 #pragma once
 #include "croft_conv_kernel.cuh"
@@ -109,6 +112,13 @@ __device__ __forceinline__ void two_conv_body(const float2* in, float2* out, con
             }
         }
     }
+}
+
+template <int N>
+__global__ void __launch_bounds__(croft_two_conv(N).w* croft_two_conv(N).t, croft_two_conv(N).minb)
+    croft_two_conv_kernel(const float2* in, float2* out, const float* g, const __grid_constant__ PassArgs A) {
+    constexpr CroftTwo K = croft_two_conv(N);
+    two_conv_body<N, K.r1, K.t, K.w, K.stage != 0>(in, out, g, A);
 }
 
 }  // namespace croft

@@ -177,6 +177,82 @@ CROFT_HD constexpr CroftTwo croft_two_row(int n) {
     }
 }
 
+// The fused convolution pass (croft_two_conv_kernel.cuh), x axis of n x 512 x 512; GB/s of its 20 bytes a
+// point (grid in and out, G in) of the three-stage kernel it replaced -> of this one.  Chosen for the long strides
+// of an x axis, the usual last axis; a 2D grid's y axis takes the same tiles.
+CROFT_HD constexpr CroftTwo croft_two_conv(int n) {
+    switch (n) {
+        case 36: return CroftTwo{6, 6, 32, 10, 1, 0};  // 5120 -> 6546
+        case 40: return CroftTwo{5, 8, 32, 8, 1, 0};  // 4876 -> 6460
+        case 45: return CroftTwo{5, 9, 32, 7, 0, 0};  // 4602 -> 6306
+        case 48: return CroftTwo{12, 4, 32, 10, 1, 0};  // 5120 -> 6592
+        case 50: return CroftTwo{10, 10, 32, 5, 1, 0};  // 4129 -> 6006
+        case 54: return CroftTwo{9, 9, 32, 6, 1, 0};  // 4189 -> 6413
+        case 60: return CroftTwo{5, 5, 32, 8, 1, 0};  // 4800 -> 6486
+        case 64: return CroftTwo{8, 8, 32, 8, 0, 0};  // 4814 -> 5479
+        case 72: return CroftTwo{8, 9, 32, 6, 0, 0};  // 4496 -> 6491
+        case 75: return CroftTwo{15, 5, 32, 6, 0, 0};  // 4915 -> 6234
+        case 80: return CroftTwo{10, 10, 32, 6, 1, 0};  // 4995 -> 6269
+        case 81: return CroftTwo{9, 9, 16, 13, 0, 0};  // 4822 -> 5182
+        case 90: return CroftTwo{10, 9, 32, 5, 0, 0};  // 4189 -> 6101
+        case 96: return CroftTwo{12, 8, 32, 5, 1, 0};  // 4551 -> 6213
+        case 100: return CroftTwo{10, 10, 32, 4, 0, 0};  // 4129 -> 5826
+        case 108: return CroftTwo{9, 9, 32, 4, 0, 0};  // 4320 -> 5928
+        case 120: return CroftTwo{15, 8, 32, 4, 1, 0};  // 4954 -> 5800
+        case 125: return CroftTwo{25, 5, 32, 4, 0, 0};  // 4324 -> 5787
+        case 128: return CroftTwo{16, 8, 32, 4, 0, 0};  // 4819 -> 6125
+        case 135: return CroftTwo{15, 9, 32, 3, 0, 0};  // 4488 -> 5531
+        case 144: return CroftTwo{16, 9, 32, 3, 0, 0};  // 4666 -> 5703
+        case 150: return CroftTwo{15, 10, 32, 3, 0, 0};  // 4364 -> 5623
+        case 160: return CroftTwo{16, 10, 32, 3, 0, 0};  // 4357 -> 5786
+        case 162: return CroftTwo{18, 9, 32, 3, 0, 0};  // 3840 -> 5455
+        case 180: return CroftTwo{10, 10, 16, 5, 1, 0};  // 4151 -> 5122
+        case 192: return CroftTwo{8, 8, 32, 2, 0, 0};  // 4551 -> 5243
+        case 200: return CroftTwo{8, 8, 16, 5, 0, 0};  // 4063 -> 5118
+        case 216: return CroftTwo{9, 9, 32, 2, 0, 0};  // 4254 -> 5127
+        case 225: return CroftTwo{15, 15, 16, 4, 1, 0};  // 4299 -> 4911
+        case 240: return CroftTwo{12, 12, 16, 3, 1, 0};  // 4690 -> 5090
+        case 243: return CroftTwo{9, 9, 16, 4, 1, 0};  // 4290 -> 4829
+        case 250: return CroftTwo{10, 10, 32, 2, 0, 0};  // 3404 -> 4872
+        case 256: return CroftTwo{16, 16, 16, 3, 0, 0};  // 4458 -> 5094
+        case 270: return CroftTwo{18, 18, 16, 3, 0, 0};  // 3456 -> 4929
+        case 288: return CroftTwo{12, 12, 16, 3, 0, 0};  // 3723 -> 5138
+        case 300: return CroftTwo{12, 12, 16, 3, 0, 0};  // 3623 -> 4868
+        case 320: return CroftTwo{20, 20, 16, 3, 1, 0};  // 3562 -> 4998
+        case 324: return CroftTwo{12, 12, 16, 3, 0, 0};  // 3560 -> 4963
+        case 360: return CroftTwo{24, 24, 16, 2, 0, 0};  // 3777 -> 4674
+        case 375: return CroftTwo{25, 25, 16, 2, 0, 0};  // 3582 -> 4358
+        case 384: return CroftTwo{24, 24, 16, 2, 0, 0};  // 3855 -> 4872
+        case 400: return CroftTwo{25, 25, 16, 2, 0, 0};  // 3821 -> 4630
+        case 405: return CroftTwo{27, 27, 16, 2, 0, 0};  // 3716 -> 4496
+        case 432: return CroftTwo{27, 27, 16, 2, 1, 0};  // 3908 -> 4718
+        case 450: return CroftTwo{25, 18, 16, 2, 1, 0};  // 3282 -> 4348
+        case 480: return CroftTwo{30, 16, 16, 2, 1, 0};  // 3913 -> 4584
+        case 486: return CroftTwo{27, 27, 16, 2, 0, 0};  // 3232 -> 4403
+        case 500: return CroftTwo{20, 25, 16, 2, 0, 0};  // 3026 -> 4216
+        case 512: return CroftTwo{32, 16, 16, 2, 0, 0};  // 3552 -> 4630
+        case 540: return CroftTwo{20, 27, 16, 2, 1, 0};  // 2999 -> 3689
+        case 576: return CroftTwo{24, 24, 16, 2, 1, 0};  // 2949 -> 3817
+        case 600: return CroftTwo{25, 25, 16, 2, 0, 0};  // 2699 -> 3638
+        case 625: return CroftTwo{25, 25, 16, 1, 1, 0};  // 2716 -> 3204
+        case 640: return CroftTwo{32, 32, 16, 1, 1, 0};  // 2801 -> 3569
+        case 648: return CroftTwo{24, 27, 16, 1, 1, 0};  // 2751 -> 3520
+        case 675: return CroftTwo{27, 27, 16, 1, 1, 0};  // 2789 -> 3333
+        case 720: return CroftTwo{24, 30, 16, 1, 1, 0};  // 2864 -> 3577
+        case 729: return CroftTwo{27, 27, 16, 1, 1, 0};  // 2732 -> 3390
+        case 750: return CroftTwo{30, 30, 16, 1, 1, 0};  // 2747 -> 3340
+        case 768: return CroftTwo{32, 32, 16, 1, 1, 0};  // 2819 -> 3700
+        case 800: return CroftTwo{32, 32, 16, 1, 1, 0};  // 2672 -> 3618
+        case 810: return CroftTwo{30, 30, 16, 1, 1, 0};  // 2665 -> 3492
+        case 864: return CroftTwo{27, 32, 16, 1, 1, 0};  // 2761 -> 3630
+        case 900: return CroftTwo{30, 30, 16, 1, 1, 0};  // 2672 -> 3482
+        case 960: return CroftTwo{32, 32, 16, 1, 1, 0};  // 2465 -> 3645
+        case 1024: return CroftTwo{32, 32, 16, 1, 0, 0};  // 2532 -> 3715
+        default: return CroftTwo{0, 0, 0, 0, 0, 0};
+    }
+}
+CROFT_HD constexpr int croft_two_conv_smem(const CroftTwo& k, int n) { return ((k.stage ? (n + 1) / 2 * 2 : 0) + k.w * n) * 8 + k.w * n * 4; }
+
 // Shared memory: [twiddles when staged][tile].
 CROFT_HD constexpr int croft_two_pad(int n) { return (n + 1) / 2 * 2; }
 CROFT_HD constexpr int croft_two_smem(const CroftTwo& k, int n, bool row) {

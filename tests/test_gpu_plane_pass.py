@@ -51,7 +51,7 @@ def test_every_length_as_y_and_z(croft_lib, n):
         _check(croft_lib, (1, n, n))
 
 
-@pytest.mark.parametrize("shape", [(160, 100, 100), (180, 75, 128), (180, 128, 75), (160, 72, 125), (625, 48, 40)])
+@pytest.mark.parametrize("shape", [(300, 100, 100), (288, 75, 128), (288, 128, 75), (300, 72, 125), (625, 48, 40)])
 def test_many_planes(croft_lib, shape):
     _check(croft_lib, shape)
 
@@ -65,7 +65,7 @@ def test_convolution_and_rule(croft_lib):
         y = p.convolve(torch.from_numpy(x).cuda(), torch.from_numpy(g).cuda())
         torch.cuda.synchronize()
     assert oracle.rel_l2(y.cpu().numpy(), oracle.convolve(x, g)) <= 4e-6 * math.log2(x.size)
-    for shape, takes in (((64, 64, 64), True), ((64, 72, 64), False), ((162, 72, 64), True), ((162, 108, 108), False),
+    for shape, takes in (((64, 64, 64), True), ((64, 72, 64), False), ((288, 72, 64), True), ((162, 72, 64), False), ((300, 108, 108), False),
                          ((8, 30, 32), False), ((8, 32, 256), False)):
         with croft_lib.Plan(*shape) as p:
             assert ("z+y in one pass" in p.describe()) == takes, shape

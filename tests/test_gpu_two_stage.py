@@ -54,3 +54,21 @@ def test_long_strides(croft_lib, n):
     x, y = x.reshape(n, -1), y.reshape(n, -1)
     pick = np.r_[0:20, 16380:16390, x.shape[1] - 20:x.shape[1]]
     _check(x[:, pick], y[:, pick], 0, -1)
+
+
+@pytest.mark.parametrize("n", [36, 108, 125, 256, 243, 360, 512, 625, 1024])
+def test_convolution_with_ragged_tiles(croft_lib, n):
+    # 135 columns of the fused axis (x; y of a 2D grid), the last tile partly filled
+    for shape in ((n, 5, 27), (1, n, 135)):
+        rng = np.random.default_rng(n)
+        x = (rng.uniform(-1, 1, shape) + 1j * rng.uniform(-1, 1, shape)).astype(np.complex64)
+        g = rng.uniform(0.1, 1, shape).astype(np.float32)
+        with croft_lib.Plan(*shape) as p:
+            assert "fwd*G*bwd fused" in p.describe()
+            d = torch.from_numpy(x).cuda()
+            y = p.convolve(d, torch.from_numpy(g).cuda())
+            p.convolve(d, torch.from_numpy(g).cuda(), d)  # in place
+            torch.cuda.synchronize()
+        assert torch.equal(torch.view_as_real(y), torch.view_as_real(d))
+        e = oracle.rel_l2(y.cpu().numpy(), oracle.convolve(x, g))
+        assert e <= 4e-6 * math.log2(x.size), (shape, e)
