@@ -331,6 +331,73 @@ template <int A, int B, class C> struct DftSplit {
         }
     }
 };
+// ---------------------------------------------------------------------------
+// power-of-two radices as fused multiply-add butterflies (complex128)
+// ---------------------------------------------------------------------------
+
+// A radix-R butterfly of a stage with P > 1 needs the DFT of w^j v[j] (w = exp(-2 pi i k / (P R))).  By decimation in
+// time, DFT_R = E[m] + (w W_R^m) O[m], E[m] - (w W_R^m) O[m] with E over the even j and O over the odd j, both with
+// w^2 in the place of w: the stage's twiddles merge with the inner ones.  A factor is taken as
+//     f = (-i)^q s (1 + i r),   q the nearest quarter turn, s = cos, r = -tan of the rest (|r| <= 1),
+// (Linzer and Feig 1993 factor the rotation like this) and one radix-2 butterfly is
+//     b1 = (-i)^q b (selects and sign bits),  b2 = b1 + i r b1,  a + s b2,  a - s b2:
+// 6 multiply-adds whatever f, each result two roundings from its operands, against 8 instructions and three
+// roundings for product, then sum and difference.  The factors of m and m + R/4 differ by -i, so R/2 factors are
+// read instead of R - 1.  Radix 16 with twiddles: 192 instructions against 228, radix 8: 72 against 84.  The
+// complex128 passes take these butterflies, being bound by the FP64 pipe (about 2 instructions per SM clock,
+// everything else idles): 128^3 109 -> 92 us a pass, 256^3 797 -> 680; rounding error of a 128-point row 1.67e-16 ->
+// 1.58e-16, of 1024 points 2.04e-16 -> 1.95e-16 (against 80 bits and more).  A stage without twiddles keeps the split butterflies: with constant factors in this form
+// radix 16 would take 148 instructions instead of 168 (128^3 88 us a pass instead of 92), but its rounding error grows
+// by 6 %, two rounded constants standing for every factor.
+//
+// Table order: level n = R, R/2, .., 2, for each the factors w^{R/n} W_n^m, m < max(1, n/4), as (s, r) with q in the
+// top two bits of s, which are 0 in a number of [0.7, 1].
+constexpr int fma_twiddle_offset(int R, int n) { return n == R ? 0 : fma_twiddle_offset(R, 2 * n) + (2 * n / 4 > 0 ? 2 * n / 4 : 1); }
+
+// (-i)^q b, q in bits 31 and 30 of `q`.
+__device__ __forceinline__ double2 quarter_turns(double2 b, int q) {
+    const bool swap = (q & 0x40000000) != 0;
+    const int fx = q & 0x80000000, fy = (q ^ (q << 1)) & 0x80000000;
+    const int xh = __double2hiint(b.x), xl = __double2loint(b.x), yh = __double2hiint(b.y), yl = __double2loint(b.y);
+    return make_double2(__hiloint2double((swap ? yh : xh) ^ fx, swap ? yl : xl),
+                        __hiloint2double((swap ? xh : yh) ^ fy, swap ? xl : yl));
+}
+// a, b -> a + f b, a - f b with f = s (1 + i r) after b's quarter turns.
+__device__ __forceinline__ void fma_butterfly(double2& a, double2& b, double s, double r) {
+    const double2 c = make_double2(fma(-r, b.y, b.x), fma(r, b.x, b.y));
+    b = make_double2(fma(-s, c.x, a.x), fma(-s, c.y, a.y));
+    a = make_double2(fma(s, c.x, a.x), fma(s, c.y, a.y));
+}
+
+// The n-point level of a radix-R butterfly: v[0], v[STRIDE], .. -> out[0 .. n-1].
+template <int R, int N, int STRIDE> struct FmaLevel {
+    __device__ __forceinline__ static void run(const double2* v, double2* out, const double2* w) {
+        double2 e[N / 2], o[N / 2];
+        FmaLevel<R, N / 2, 2 * STRIDE>::run(v, e, w);
+        FmaLevel<R, N / 2, 2 * STRIDE>::run(v + STRIDE, o, w);
+        for_each_index<N / 2>([&](auto mc) {
+            constexpr int m = decltype(mc)::value;
+            constexpr bool turned = N >= 4 && m >= N / 4;  // factor of m - N/4 times -i
+            const double2 f = w[fma_twiddle_offset(R, N) + (turned ? m - N / 4 : m)];
+            const int hi = __double2hiint(f.x);
+            double2 a = e[m], b = quarter_turns(turned ? mul_mi(o[m]) : o[m], hi);
+            fma_butterfly(a, b, __hiloint2double(hi & 0x3fffffff, __double2loint(f.x)), f.y);
+            out[m] = a;
+            out[m + N / 2] = b;
+        });
+    }
+};
+template <int R, int STRIDE> struct FmaLevel<R, 1, STRIDE> {
+    __device__ __forceinline__ static void run(const double2* v, double2* out, const double2*) { out[0] = v[0]; }
+};
+// v[0 .. R-1] -> the DFT of w^j v[j], f the R/2 factors.
+template <int R> __device__ __forceinline__ void fma_dft(double2* v, const double2* f) {
+    double2 out[R];
+    FmaLevel<R, R, 1>::run(v, out, f);
+#pragma unroll
+    for (int j = 0; j < R; ++j) v[j] = out[j];
+}
+
 template <class C> struct Dft<6, C> : DftSplit<3, 2, C> {};
 template <class C> struct Dft<10, C> : DftSplit<5, 2, C> {};
 template <class C> struct Dft<12, C> : DftSplit<4, 3, C> {};

@@ -102,18 +102,13 @@ __device__ __forceinline__ void conv_middle(const Src& src, const Mid& mid, cons
     for (int q = 0; q < QM; ++q) {
         const int b = lane + q * T;
         if (ok && (NB % T == 0 || b < NB)) {
-            if (P > 1) {
-                const C* w = stw + (P - 1) + b;
-#pragma unroll
-                for (int j = 1; j < RAD; ++j) v[q][j] = cmul(v[q][j], w[(j - 1) * P]);
-            }
-            dft<RAD>(v[q]);
+            stage_dft<RAD, P>(v[q], stw + (P - 1) + b);
 #pragma unroll
             for (int j = 0; j < RAD; ++j) {
                 const R ga = gcol[(b + j * P) * W];
                 v[q][j] = mkc<C>(v[q][j].x * ga, -(v[q][j].y * ga));
             }
-            dft<RAD>(v[q]);
+            stage_dft<RAD, 1>(v[q], stw);
 #pragma unroll
             for (int j = 0; j < RAD; ++j) dst.store(b * RAD + j, v[q][j]);
         }

@@ -28,6 +28,14 @@ namespace croft {
 // Accessors are templates on the complex type C (float2 or double2); the
 // float2 names below are the complex64 instances.
 
+// Conjugates v when isign = -1.  (complex128: by the sign bit, on the integer pipe; a multiply by isign
+// at the load and at the store is 2 of the 23 instructions a point of a 128-point pass on the FP64 pipe.)
+__device__ __forceinline__ void conj_if(float2& v, float isign) { v.y *= isign; }
+__device__ __forceinline__ void conj_if(double2& v, float isign) {
+    const int flip = __float_as_int(isign) & 0x80000000;
+    v.y = __hiloint2double(__double2hiint(v.y) ^ flip, __double2loint(v.y));
+}
+
 // Pencil in HBM with element stride `stride`; conj() on the way in/out when isign = -1.
 template <class C>
 struct GlobalInT {
@@ -37,7 +45,7 @@ struct GlobalInT {
     float isign;
     __device__ __forceinline__ C load(int a) const {
         C t = p[(long long)a * stride];
-        t.y *= isign;
+        conj_if(t, isign);
         return t;
     }
 };
@@ -48,7 +56,7 @@ struct GlobalInUnitT {  // unit stride (contiguous pencil)
     float isign;
     __device__ __forceinline__ C load(int a) const {
         C t = p[a];
-        t.y *= isign;
+        conj_if(t, isign);
         return t;
     }
 };
@@ -72,7 +80,7 @@ struct GlobalOutT {
     long long stride;
     float isign;
     __device__ __forceinline__ void store(int a, C v) const {
-        v.y *= isign;
+        conj_if(v, isign);
         p[(long long)a * stride] = v;
     }
 };
@@ -82,7 +90,7 @@ struct GlobalOutUnitT {
     C* p;
     float isign;
     __device__ __forceinline__ void store(int a, C v) const {
-        v.y *= isign;
+        conj_if(v, isign);
         p[a] = v;
     }
 };
@@ -187,6 +195,25 @@ struct PairSwapStores : std::false_type {};
 template <class D>
 struct PairSwapStores<D, std::void_t<decltype(D::kPairSwap)>> : std::bool_constant<D::kPairSwap> {};
 
+// The radix-R DFT of a stage-P butterfly's inputs after their twiddles (w: stw + P - 1 + k; entry i at w[i * P]).
+// complex128 with a power-of-two radix: fused multiply-add butterflies, whose table holds the R/2 merged
+// factors in the place of the R - 1 powers (build_twiddles64).
+template <int R, int P, class C>
+__device__ __forceinline__ void stage_dft(C* v, const C* w) {
+    if constexpr (P == 1) {
+        dft<R>(v);
+    } else if constexpr (sizeof(C) == 16 && (R & (R - 1)) == 0) {
+        C f[R / 2];
+#pragma unroll
+        for (int i = 0; i < R / 2; ++i) f[i] = w[i * P];
+        fma_dft<R>(v, f);
+    } else {
+#pragma unroll
+        for (int j = 1; j < R; ++j) v[j] = cmul(v[j], w[(j - 1) * P]);
+        dft<R>(v);
+    }
+}
+
 template <class SchedT, int S, int T, class Src, class Mid, class Dst>
 __device__ __forceinline__ void fft_stage_s(const Src& src, const Mid& mid, const Dst& dst,
                                             const typename Src::value_type* stw, int lane, bool ok) {
@@ -212,12 +239,7 @@ __device__ __forceinline__ void fft_stage_s(const Src& src, const Mid& mid, cons
         const int b = lane + q * T;
         if (ok && (NB % T == 0 || b < NB)) {
             const int k = (P == 1) ? 0 : b % P;
-            if (P > 1) {
-                const C* w = stw + (P - 1) + k;
-#pragma unroll
-                for (int j = 1; j < R; ++j) v[q][j] = cmul(v[q][j], w[(j - 1) * P]);
-            }
-            dft<R>(v[q]);
+            stage_dft<R, P>(v[q], stw + (P - 1) + k);
             const int o = (b - k) * R + k;
             if constexpr (P == 1 && R % 2 == 0 && PairSwapStores<Dst>::value) {
                 // same stores, odd butterflies take each pair (j, j+1) in swapped order: the

@@ -64,20 +64,44 @@ static void twiddle64(long long r, long long N, double* re, double* im) {
     *im = y;
 }
 
-// The same table in double precision (complex128 plans).
+// The table of complex128 plans, in double precision: the same layout, entry i, k of the stage with radix R after sub-transforms
+// of length p at p - 1 + i*p + k; where R is a power of two, i < R/2 counts the merged factors of the
+// multiply-add butterflies (croft_butterflies.cuh): per level m = R, R/2, .., 2, w_{pR}^{k R/m} W_m^q for q < max(1, m/4),
+// each as (cos, -tan) of what is left after the nearest quarter turns, whose number sits in the top bits of the cosine.
+static void merged_factor64(long long num, long long den, double* s, double* r) {
+    num = ((num % den) + den) % den;
+    const int q = (int)((8 * num + den) / (2 * den)) & 3;  // nearest quarter turn
+    long long rest = 4 * num - q * den;                    // of the angle, in units of a quarter turn / den
+    if (2 * rest > den) rest -= 4 * den;                   // (the last eighth of the circle belongs to q = 0)
+    const double ph = (M_PI / 2.0) * (double)rest / (double)den;
+    const double c = cos(ph);
+    unsigned long long bits;
+    memcpy(&bits, &c, sizeof(bits));
+    bits |= (unsigned long long)q << 62;
+    memcpy(s, &bits, sizeof(bits));
+    *r = -tan(ph);
+}
 static int build_twiddles64(int n, const int* radices, int ns, double* out) {
     int p = 1;
     for (int s = 0; s < ns; ++s) {
         int R = radices[s];
         if (R < 2 || p * R > n) return -1;
-        for (int j = 1; j < R; ++j)
-            for (int k = 0; k < p; ++k) {
-                double re, im;
-                twiddle64((long long)j * k, (long long)p * R, &re, &im);
-                long long idx = (long long)(p - 1) + (long long)(j - 1) * p + k;
-                out[2 * idx] = re;
-                out[2 * idx + 1] = im;
-            }
+        const long long den = (long long)p * R;
+        if ((R & (R - 1)) == 0) {
+            int i = 0;
+            for (int m = R; m >= 2; m /= 2)
+                for (int q = 0; q < (m >= 4 ? m / 4 : 1); ++q, ++i)
+                    for (int k = 0; k < p; ++k) {
+                        const long long idx = (long long)(p - 1) + (long long)i * p + k;
+                        merged_factor64((long long)k * (R / m) + (long long)p * (R / m) * q, den, &out[2 * idx], &out[2 * idx + 1]);
+                    }
+        } else {
+            for (int j = 1; j < R; ++j)
+                for (int k = 0; k < p; ++k) {
+                    const long long idx = (long long)(p - 1) + (long long)(j - 1) * p + k;
+                    twiddle64((long long)j * k % den, den, &out[2 * idx], &out[2 * idx + 1]);
+                }
+        }
         p *= R;
     }
     return p == n ? n - 1 : -1;
