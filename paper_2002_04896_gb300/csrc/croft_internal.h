@@ -110,6 +110,7 @@ struct TwoLaunch {
     const float2* tw;  // w_n^{jk} at [j * r1 + k]
     CroftColDiv cdiv;  // for this tile width
     int r1, T, W, grid, block, smem;
+    int ctas;          // that share a tile
 };
 
 struct PassLaunch {

@@ -229,7 +229,7 @@ void shape_two(TwoLaunch& two, int layout, int n, long long M, long long ncols) 
     if (!f) f = lookup_two_kernel_group_3(layout, n, lng);
     if (!f) return;
     const int smem = croft_two_smem(K, n, row);
-    const long long grid = (ncols + K.w - 1) / K.w;
+    const long long grid = (ncols + K.w - 1) / K.w * K.ctas;
     if (smem > g_max_smem || grid > 0x7fffffffLL) return;
     if (smem > 48 * 1024 && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
         cudaGetLastError();
@@ -239,6 +239,7 @@ void shape_two(TwoLaunch& two, int layout, int n, long long M, long long ncols) 
     two.r1 = K.r1;
     two.T = K.t;
     two.W = K.w;
+    two.ctas = K.ctas;
     two.grid = (int)grid;
     two.block = K.w * K.t;
     two.smem = smem;

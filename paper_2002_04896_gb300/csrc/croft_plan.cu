@@ -241,11 +241,8 @@ static croft_status attach_two(croft_plan p, int axis, PassLaunch& L) {
     if (!L.two.fn) return CROFT_OK;
     const int n = L.args.n;
     L.two.tw = p->tw_dev[axis] + n;  // (the axis's second table)
-    std::vector<float> tw(2 * (size_t)n);
-    host_build_two_twiddles(n, L.two.r1, tw.data());
-    return cudaMemcpy((void*)L.two.tw, tw.data(), sizeof(float2) * (size_t)n, cudaMemcpyHostToDevice) == cudaSuccess
-               ? CROFT_OK
-               : CROFT_ERR_CUDA;
+    host_build_two_twiddles(n, L.two.r1, p->tw_host[axis].data() + 2 * (size_t)n);
+    return CROFT_OK;
 }
 
 static croft_status add_axis_pass(croft_plan p, int axis, int x0 = 0, int nxs = -1, int group = -1, int src_in = -1) {
@@ -406,10 +403,7 @@ static croft_status plan_zy(croft_plan p) {
     }
     for (int axis = 1; axis <= 2; ++axis) {
         const int n = p->dims[axis];
-        std::vector<float> tw(2 * (size_t)n);
-        host_build_two_twiddles(n, croft_plane_r1(n), tw.data());
-        if (cudaMemcpy(p->tw_dev[axis] + 2 * n, tw.data(), sizeof(float2) * (size_t)n, cudaMemcpyHostToDevice) != cudaSuccess)
-            return CROFT_ERR_CUDA;
+        host_build_two_twiddles(n, croft_plane_r1(n), p->tw_host[axis].data() + 4 * (size_t)n);
     }
     z.args.tw_z = p->tw_dev[2] + 2 * nz;
     z.args.tw_y = p->tw_dev[1] + 2 * ny;
@@ -448,6 +442,17 @@ static croft_status add_plane_pass(croft_plan p, const PlaneKernel* pk) {
     return CROFT_OK;
 }
 
+// The complex64 tables of every axis, in one copy each.
+static croft_status upload_tables(croft_plan p) {
+    for (int a = 0; a < 3; ++a) {
+        std::vector<float>& t = p->tw_host[a];
+        if (!t.empty() && cudaMemcpy(p->tw_dev[a], t.data(), sizeof(float) * t.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+            return CROFT_ERR_CUDA;
+        std::vector<float>().swap(t);
+    }
+    return CROFT_OK;
+}
+
 // Fused convolution pass for croft_exec_convolve: it replaces the plan's last pass
 // when that pass is a plain (CUDA-core, non-pipelined) axis pass over the whole grid
 // that forms a logical pass of its own; otherwise convolve runs F, multiply, B.
@@ -466,7 +471,7 @@ static void plan_conv(croft_plan p) {
     const long long M = (axis == 2) ? 1 : (axis == 1 ? (long long)p->dims[2] : (long long)p->dims[1] * p->dims[2]);
     if (f64 ? !conv64_kernel_for(n) : !conv_kernel_for(n)) return;
     PassLaunch L;
-    const CroftTwo K = f64 ? CroftTwo{0, 0, 0, 0, 0, 0} : croft_two_conv(n);
+    const CroftTwo K = f64 ? CroftTwo{0, 0, 0, 0, 0, 0, 0} : croft_two_conv(n);
     if (K.r1) {  // two stages (croft_two_conv_kernel.cuh)
         memset(&L, 0, sizeof(L));
         const long long ncols = N / n, grid = (ncols + K.w - 1) / K.w;
@@ -482,14 +487,8 @@ static void plan_conv(croft_plan p) {
         L.block = K.w * K.t;
         L.smem = croft_two_conv_smem(K, n);
         if (L.smem > g_max_smem) return;
-        std::vector<float> tw(2 * (size_t)n);
-        host_build_two_twiddles(n, K.r1, tw.data());
-        float2* d = p->tw_dev[axis] + 3 * n;  // (the axis's fourth table)
-        if (cudaMemcpy(d, tw.data(), sizeof(float2) * (size_t)n, cudaMemcpyHostToDevice) != cudaSuccess) {
-            cudaGetLastError();
-            return;
-        }
-        L.args.tw = d;
+        host_build_two_twiddles(n, K.r1, p->tw_host[axis].data() + 6 * (size_t)n);
+        L.args.tw = p->tw_dev[axis] + 3 * n;  // (the axis's fourth table)
     } else {
         // the general kernel runs the column schedule on the axis's own twiddle table
         const CroftSched sa = croft_pass_sched_v(n, Lp.layout, f64 ? 16 : 8, Lp.sv),
@@ -636,12 +635,10 @@ static croft_status create_impl(croft_plan* out, int nx, int ny, int nz, croft_d
                 return fail(p, CROFT_ERR_CUDA);
             continue;
         }
-        std::vector<float> tw(2 * (size_t)(n - 1) + 2, 0.f);
-        if (build_twiddles(n, rad, ns, tw.data()) != n - 1) return fail(p, CROFT_ERR_UNSUPPORTED_SIZE);
-        // (room for three more tables behind it: attach_two, plan_zy, plan_conv)
+        // (room for three more tables behind it: attach_two, plan_zy, plan_conv; upload_tables copies all four)
+        p->tw_host[axis].assign(8 * (size_t)n, 0.f);
+        if (build_twiddles(n, rad, ns, p->tw_host[axis].data()) != n - 1) return fail(p, CROFT_ERR_UNSUPPORTED_SIZE);
         if (dev_alloc((void**)&p->tw_dev[axis], sizeof(float2) * 4 * (size_t)n) != cudaSuccess) return fail(p, CROFT_ERR_OOM);
-        if (cudaMemcpy(p->tw_dev[axis], tw.data(), sizeof(float2) * (size_t)(n - 1), cudaMemcpyHostToDevice) != cudaSuccess)
-            return fail(p, CROFT_ERR_CUDA);
     }
 
     // schedule: fused yz-plane pass + x pass when a plane kernel exists for (ny, nz)
@@ -676,6 +673,7 @@ static croft_status create_impl(croft_plan* out, int nx, int ny, int nz, croft_d
         croft_status st = add_slab_passes(p, planes);
         if (st != CROFT_OK) return fail(p, st);
         plan_conv(p);
+        if (upload_tables(p) != CROFT_OK) return fail(p, CROFT_ERR_CUDA);
         *out = p;
         return CROFT_OK;
     }
@@ -693,6 +691,7 @@ static croft_status create_impl(croft_plan* out, int nx, int ny, int nz, croft_d
         if (st != CROFT_OK) return fail(p, st);
     }
     plan_conv(p);
+    if (upload_tables(p) != CROFT_OK) return fail(p, CROFT_ERR_CUDA);
     const char* log = getenv("CROFT_LOG");
     if (log && log[0] == '1') {
         char buf[2048];
@@ -985,8 +984,8 @@ int croft_plan_describe(croft_plan plan, char* buf, int cap) {
         snprintf(tmp, sizeof(tmp), " T=%d W=%d block=%d grid=%d smem=%d", L.T, L.args.W, L.block, L.grid, L.smem);
         s += tmp;
         if (L.two.fn) {  // the kernel that runs in its place
-            snprintf(tmp, sizeof(tmp), " -> two-stage %dx%d T=%d W=%d block=%d grid=%d smem=%d", L.two.r1, L.args.n / L.two.r1,
-                     L.two.T, L.two.W, L.two.block, L.two.grid, L.two.smem);
+            snprintf(tmp, sizeof(tmp), " -> two-stage%s %dx%d T=%d W=%d block=%d grid=%d smem=%d",
+                     L.two.ctas == 2 ? " by two CTAs" : "", L.two.r1, L.args.n / L.two.r1, L.two.T, L.two.W, L.two.block, L.two.grid, L.two.smem);
             s += tmp;
         }
     }

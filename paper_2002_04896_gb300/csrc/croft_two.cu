@@ -12,13 +12,18 @@
 
 namespace croft {
 
+template <int N, bool LONG>
+static pass_fn two_col_at() {
+    if constexpr (croft_two_col(N, LONG).ctas == 2) return croft_two_pair_kernel<N, LONG>;
+    else if constexpr (croft_two_col(N, LONG).r1 != 0) return croft_two_col_kernel<N, LONG>;
+    else return nullptr;
+}
 template <int N>
 static pass_fn two_col(bool long_stride) {
-    if constexpr (croft_two_col(N, true).r1 != 0 && croft_two_split_by_stride(N)) {
-        if (long_stride) return croft_two_col_kernel<N, true>;
+    if constexpr (croft_two_split_by_stride(N)) {
+        if (long_stride) return two_col_at<N, true>();
     }
-    if constexpr (croft_two_col(N, false).r1 != 0) return croft_two_col_kernel<N, false>;
-    else return nullptr;
+    return two_col_at<N, false>();
 }
 
 template <int N>

@@ -122,6 +122,80 @@ __device__ __forceinline__ const float2* two_twiddles(const float2* tw, float2* 
     }
 }
 
+// The column pass of long axes: one tile of W columns shared by a cluster of two CTAs.  CTA r takes the stage-1
+// butterflies b of its half and the stage-2 butterflies k of its half; element (b, k) goes straight into the shared
+// memory of the CTA that needs it (half of the stores through distributed shared memory), [b][k - its first k][column].
+// Barriers: the first (arrived at entry) tells that the partner runs before anything is stored into its
+// memory; the second publishes the stores.  No CTA touches its partner's memory after that, so either may
+// leave, and both have read their rows of the tile before either writes (in place).
+// What bounds it: the latency of a round at three or four CTAs of about 250 threads per SM, 5.0-5.5 TB/s across megabytes
+// (the 16-column tile in one CTA of its own per SM: 4.4-4.9).
+template <int N, bool LONG>
+__global__ void __cluster_dims__(2, 1, 1)
+    __launch_bounds__(croft_two_col(N, LONG).w* croft_two_col(N, LONG).t, croft_two_col(N, LONG).minb)
+    croft_two_pair_kernel(const float2* in, float2* out, const __grid_constant__ PassArgs A) {
+    constexpr CroftTwo K = croft_two_col(N, LONG);
+    constexpr int R1 = K.r1, R2 = N / R1, T = K.t, W = K.w;
+    constexpr int H1 = (R2 + 1) / 2, H2 = (R1 + 1) / 2;  // butterflies of CTA 0 in the two stages
+    constexpr int Q1 = (H1 + T - 1) / T, Q2 = (H2 + T - 1) / T;
+    namespace cg = cooperative_groups;
+    extern __shared__ __align__(16) float2 two_smem[];
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int r = (int)cluster.block_rank();
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    pdl_allow_dependents();
+    pdl_wait();
+    const int c = threadIdx.x % W, lane = threadIdx.x / W;
+    const long long col = (long long)(blockIdx.x / 2) * W + c;
+    const bool ok = col < A.ncols;
+    long long b_, m_;
+    col_split(col, A, b_, m_);
+    const long long base = b_ * (long long)N * A.M + m_;
+    {
+        const GlobalIn src{in + base, A.M, A.isign};
+        float2 v[Q1][R1];
+#pragma unroll
+        for (int q = 0; q < Q1; ++q) {
+            const int lb = lane + q * T, b = r * H1 + lb;
+            if (ok && lb < H1 && b < R2) {
+#pragma unroll
+                for (int j = 0; j < R1; ++j) v[q][j] = src.load(b + j * R2);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < Q1; ++q) dft<R1>(v[q]);
+        asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+        float2* first = (r == 0 ? two_smem : cluster.map_shared_rank(two_smem, 0)) + c;
+        float2* second = (r == 1 ? two_smem : cluster.map_shared_rank(two_smem, 1)) + c;
+#pragma unroll
+        for (int q = 0; q < Q1; ++q) {
+            const int lb = lane + q * T, b = r * H1 + lb;
+            if (lb < H1 && b < R2) {
+#pragma unroll
+                for (int j = 0; j < R1; ++j) (j < H2 ? first : second)[(b * H2 + (j < H2 ? j : j - H2)) * W] = v[q][j];
+            }
+        }
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    const GlobalOut dst{out + base, A.M, A.isign};
+#pragma unroll
+    for (int q = 0; q < Q2; ++q) {
+        const int lk = lane + q * T, k = r * H2 + lk;
+        if (lk < H2 && k < R1) {
+            float2 v[R2];
+#pragma unroll
+            for (int j = 0; j < R2; ++j) v[j] = two_smem[(j * H2 + lk) * W + c];
+#pragma unroll
+            for (int j = 1; j < R2; ++j) v[j] = cmul(v[j], A.tw[j * R1 + k]);
+            dft<R2>(v);
+            if (ok) {
+#pragma unroll
+                for (int j = 0; j < R2; ++j) dst.store(k + j * R1, v[j]);
+            }
+        }
+    }
+}
+
 // The column pass: W adjacent columns per CTA, T threads per column.  LONG: the tile for strides
 // beyond kTwoLongStride (croft_two_col).
 template <int N, bool LONG>

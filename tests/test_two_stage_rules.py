@@ -16,7 +16,7 @@ PROGRAM = r"""
 #include <cstdio>
 #include "croft_two_stage.h"
 static void put(char k, int n, const CroftTwo& t, bool row) {
-    if (t.r1) std::printf("%c %d %d %d %d %d %d %d %d\n", k, n, t.r1, t.t, t.w, t.minb, t.stage, t.ld, croft_two_smem(t, n, row));
+    if (t.r1) std::printf("%c %d %d %d %d %d %d %d %d %d\n", k, n, t.r1, t.t, t.w, t.minb, t.stage, t.ld, t.ctas, croft_two_smem(t, n, row));
 }
 int main() {
     for (int n = 1; n <= 5000; ++n) {
@@ -43,7 +43,7 @@ def table(tmp_path_factory):
 
 def test_entries_fit(table):
     assert len(table) > 100
-    for kind, n, r1, t, w, minb, stage, ld, smem in table:
+    for kind, n, r1, t, w, minb, stage, ld, ctas, smem in table:
         r2 = n // r1
         assert r1 * r2 == n and r1 in RADICES and r2 in RADICES, (kind, n)
         threads = w * t
@@ -55,3 +55,5 @@ def test_entries_fit(table):
             assert ld >= r2 * (r1 + (r1 % 2 == 0)) - (r1 % 2 == 0), (n, ld)
         else:
             assert w % 8 == 0, (kind, n, w)  # rows of at least 64 bytes
+        # two CTAs share a tile: each takes half of the butterflies of either stage, from global twiddles
+        assert ctas == 1 or (ctas == 2 and kind != "r" and stage == 0 and smem == r2 * ((r1 + 1) // 2) * w * 8)
