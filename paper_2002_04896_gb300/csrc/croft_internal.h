@@ -172,6 +172,8 @@ cudaError_t launch_plane_pass(const PlanePass& P, const float2* in, float2* out,
 // croft_tc.cu: tensor-core pass kernels (NULL when n has no instantiation); prec 0 = split
 // bf16, 1 = split fp16 with per-butterfly power-of-two scaling (TcPrec)
 pass_fn tc_pass_kernel_for(int layout, int n, int prec);
+// Launch shape of a two-stage tensor-core pass (croft_tc_two) in L; false when it does not fit.
+bool shape_tc_two(PassLaunch& L, int layout, int n, long long M, long long ncols);
 void tc_dft16_matrix(unsigned char* out4096, int prec);  // B operand (hi | lo) in the kernels' smem layout
 
 // croft_alloc.cu: all library allocations (failure injection for tests)

@@ -32,6 +32,7 @@ bool shape_pass(PassLaunch& L, int layout, int n, long long M, long long ncols, 
     A.n = n;
     A.M = M;
     A.ncols = ncols;
+    if (tc && croft_tc_two(n)) return shape_tc_two(L, layout, n, M, ncols);
     const int T = L.th > 0 ? L.th : croft_threads_per_pencil(n);
     L.T = T;
     A.tw_pad = ((n + 1) / 2) * 2;  // keeps the tile 16-byte aligned
@@ -49,7 +50,6 @@ bool shape_pass(PassLaunch& L, int layout, int n, long long M, long long ncols, 
         int W = 16;
         if (tc) {
             while (W * 2 * T <= 256) W *= 2;
-            if (croft_col_narrow(n, (int)es, M * es)) W = kColNarrowWidth;  // (two 128-butterfly groups)
         } else {
             W = croft_col_width_at(n, (int)es, M * es);  // a width the kernels are built for
         }
@@ -287,7 +287,7 @@ static cudaError_t launch_ex(void (*f)(P...), const Shape& L, cudaStream_t s, bo
     return cudaLaunchKernelEx(&cfg, f, args...);
 }
 
-bool pass_supports_pdl(const PassLaunch& L) { return !L.tc; }
+bool pass_supports_pdl(const PassLaunch& L) { return !L.tc || croft_tc_two(L.args.n); }
 
 cudaError_t prepare_pass(const PassLaunch& L) {
     if (L.kind == PASS_PLANE) {
@@ -367,8 +367,7 @@ cudaError_t launch_pass(const PassLaunch& L, const void* vin, void* vout, cudaSt
     if (L.tc) {
         pass_fn f = tc_pass_kernel_for(L.layout, L.args.n, L.tc - 1);
         if (!f) return cudaErrorInvalidValue;
-        f<<<L.grid, L.block, L.smem, s>>>(in, out, L.args);
-        return cudaGetLastError();
+        return launch_ex(f, L, s, pdl, in, out, L.args);
     }
     pass_fn f = pass_kernel_for(L.layout, L.args.n, L.args.W, L.sv, L.th);
     if (!f) return cudaErrorInvalidValue;

@@ -637,7 +637,8 @@ static croft_status create_impl(croft_plan* out, int nx, int ny, int nz, croft_d
         }
         // (room for three more tables behind it: attach_two, plan_zy, plan_conv; upload_tables copies all four)
         p->tw_host[axis].assign(8 * (size_t)n, 0.f);
-        if (build_twiddles(n, rad, ns, p->tw_host[axis].data()) != n - 1) return fail(p, CROFT_ERR_UNSUPPORTED_SIZE);
+        if (p->axis_tc[axis] && croft_tc_two(n)) host_build_two_twiddles(n, 16, p->tw_host[axis].data());
+        else if (build_twiddles(n, rad, ns, p->tw_host[axis].data()) != n - 1) return fail(p, CROFT_ERR_UNSUPPORTED_SIZE);
         if (dev_alloc((void**)&p->tw_dev[axis], sizeof(float2) * 4 * (size_t)n) != cudaSuccess) return fail(p, CROFT_ERR_OOM);
     }
 
@@ -972,7 +973,7 @@ int croft_plan_describe(croft_plan plan, char* buf, int cap) {
                  L.tc ? (L.tc == 2 ? "+tc_fp16x3" : "+tc_bf16x3") : "", L.ring ? "+ring" : (L.pair ? "+pair" : ""),
                  L.args.n);
         s += tmp;
-        CroftSched sc = L.tc ? croft_make_sched_tc(L.args.n) : croft_pass_sched_v(L.args.n, L.layout, L.f64 ? 16 : 8, L.sv);
+        CroftSched sc = L.tc ? (croft_tc_two(L.args.n) ? CroftSched{2, {16, L.args.n / 16}} : croft_make_sched_tc(L.args.n)) : croft_pass_sched_v(L.args.n, L.layout, L.f64 ? 16 : 8, L.sv);
         if (L.pair) {  // radix 2 across the pair over the half length's schedule
             sc = croft_pass_sched(L.args.n / 2, LAYOUT_COL, 8);
             s += "2|";

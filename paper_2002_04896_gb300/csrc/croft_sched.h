@@ -117,6 +117,10 @@ CROFT_HD constexpr CroftSched croft_make_sched_tc(int n) {
     return s;
 }
 
+// Whether a tensor-core pass takes two stages, 16 on the tensor cores and n / 16 on the CUDA cores
+// (croft_tc_two_kernel.cuh): lengths 32 .. 512; beyond, the second radix would exceed 32.
+CROFT_HD constexpr bool croft_tc_two(int n) { return n % 16 == 0 && n >= 32 && n <= 512; }
+
 // Length of the sub-transforms that stage `stage` combines (product of the earlier radices).
 CROFT_HD constexpr int croft_sched_p(const CroftSched& s, int stage) {
     int p = 1;

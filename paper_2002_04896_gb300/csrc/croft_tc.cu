@@ -4,6 +4,7 @@
 
 #include "croft_tc_kernel.cuh"
 #include "croft_tc_operand.h"
+#include "croft_tc_two_kernel.cuh"
 
 namespace croft {
 
@@ -19,14 +20,18 @@ namespace croft {
 #define CROFT_TCAT_(a, b) a##b
 #define CROFT_TCAT(a, b) CROFT_TCAT_(a, b)
 
+template <int N, int PREC>
+static pass_fn tc_kernel_of(int layout) {
+    if constexpr (croft_tc_two(N))
+        return layout == LAYOUT_ROW ? croft_tc_two_kernel<LAYOUT_ROW, N, PREC> : croft_tc_two_kernel<LAYOUT_COL, N, PREC>;
+    else
+        return layout == LAYOUT_ROW ? croft_pass_kernel_tc<LAYOUT_ROW, N, PREC> : croft_pass_kernel_tc<LAYOUT_COL, N, PREC>;
+}
+
 pass_fn CROFT_TCAT(lookup_tc_kernel_group_, CROFT_TC_GROUP)(int layout, int n, int prec) {
 #define CROFT_TC_CASE(N)                                                                                     \
     case N:                                                                                                  \
-        if (prec == TC_BF16X3)                                                                               \
-            return layout == LAYOUT_ROW ? croft_pass_kernel_tc<LAYOUT_ROW, N, TC_BF16X3>                     \
-                                        : croft_pass_kernel_tc<LAYOUT_COL, N, TC_BF16X3>;                    \
-        return layout == LAYOUT_ROW ? croft_pass_kernel_tc<LAYOUT_ROW, N, TC_FP16X3>                         \
-                                    : croft_pass_kernel_tc<LAYOUT_COL, N, TC_FP16X3>;
+        return prec == TC_BF16X3 ? tc_kernel_of<N, TC_BF16X3>(layout) : tc_kernel_of<N, TC_FP16X3>(layout);
     switch (n) {
         CROFT_TCAT(CROFT_TC_SIZES_, CROFT_TC_GROUP)(CROFT_TC_CASE)
         default: return nullptr;
@@ -35,6 +40,19 @@ pass_fn CROFT_TCAT(lookup_tc_kernel_group_, CROFT_TC_GROUP)(int layout, int n, i
 }
 
 #else  // the lookup and the DFT-16 operands (one translation unit)
+
+bool shape_tc_two(PassLaunch& L, int layout, int n, long long M, long long ncols) {
+    if (!croft_tc_two(n)) return false;
+    const long long grid = (ncols + tc_two_width(n) - 1) / tc_two_width(n);
+    L.T = tc_two_threads(n);
+    L.args.W = tc_two_width(n);
+    L.block = 256;
+    L.smem = tc_two_smem(n, layout == LAYOUT_ROW);
+    if (grid > 0x7fffffffLL || L.smem > g_max_smem) return false;
+    L.grid = (int)grid;
+    if (layout == LAYOUT_COL) L.args.cdiv = croft_coldiv_make(M, ncols + L.args.W);
+    return true;
+}
 
 pass_fn lookup_tc_kernel_group_0(int layout, int n, int prec);
 pass_fn lookup_tc_kernel_group_1(int layout, int n, int prec);

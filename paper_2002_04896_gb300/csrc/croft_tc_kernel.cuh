@@ -1,4 +1,6 @@
-// croft_tc_kernel.cuh - pass kernel whose first (radix-16) stage runs on the tensor cores.
+// croft_tc_kernel.cuh - pass kernel whose first (radix-16) stage runs on the tensor cores, in three or more stages: the
+// 16-point axes and those of 576 to 1024 points (32 to 512: croft_tc_two_kernel.cuh, which shares the
+// operand preparation and the instructions below).
 //
 // A radix-16 Stockham stage applies, to every butterfly b, the 16-point DFT
 // matrix F (F[k][j] = exp(-2 pi i jk/16)) after the twiddles: y = F u.  Over a
