@@ -29,7 +29,7 @@ namespace croft {
 // (complex64, the default) or double2 (complex128, twiddles from A.tw64).
 // COL kernels are specialised on the column-tile width WC as well (so the
 // shared-memory indices fold into constants); ROW kernels take W from A.W.
-template <int LAYOUT, int N, class C, int WC, int SV = 0, int TH = 0>
+template <int LAYOUT, int N, class C, int WC, bool BACK, int SV = 0, int TH = 0>
 __device__ __forceinline__ void pass_body(const C* in, C* out, const PassArgs& A) {
     constexpr int T = TH > 0 ? TH : croft_threads_per_pencil(N);  // TH: threads per pencil, if not the rule's
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -56,7 +56,7 @@ __device__ __forceinline__ void pass_body(const C* in, C* out, const PassArgs& A
         static_assert(LAYOUT == LAYOUT_ROW || WC > 0, "COL kernels need a compile-time tile width");
         const int c = threadIdx.x % WC;
         const int lane = threadIdx.x / WC;
-        const long long col = (long long)blockIdx.x * WC + c;
+        const long long col = (long long)(BACK ? col_tile(A, blockIdx.x, gridDim.x) : blockIdx.x) * WC + c;
         const bool ok = col < A.ncols;
         long long b, m;
         col_split(col, A, b, m);
@@ -75,12 +75,16 @@ __device__ __forceinline__ void pass_body(const C* in, C* out, const PassArgs& A
     }
 }
 
+// BACK: the kernel follows A.backwards (col_tile).  The kernels without a minimum of CTAs per SM - lengths of short
+// passes inside the L2 among them - do not: choosing the tile ahead of every address costs a 128^3 transform
+// 0.9 of its 19 us.
+//
 // The pass kernel.  (Its launch bound names no minimum of CTAs per SM: with an
 // explicit minimum of one, ptxas allocates far more registers - 83 instead of 52
 // for the 256-point COL kernel - and the pass slows from 46 to 60 us.)
 template <int LAYOUT, int N, class C = float2, int WC = 0>
 __global__ void __launch_bounds__(512) croft_pass_kernel(const C* in, C* out, const __grid_constant__ PassArgs A) {
-    pass_body<LAYOUT, N, C, WC>(in, out, A);
+    pass_body<LAYOUT, N, C, WC, false>(in, out, A);
 }
 
 // The same with registers bounded for MINB CTAs of MAXT threads per SM (croft_col_minb,
@@ -88,7 +92,7 @@ __global__ void __launch_bounds__(512) croft_pass_kernel(const C* in, C* out, co
 template <int LAYOUT, int N, class C, int WC, int MINB, int MAXT = 512, int SV = 0, int TH = 0>
 __global__ void __launch_bounds__(MAXT, MINB) croft_pass_kernel_bounded(const C* in, C* out,
                                                                          const __grid_constant__ PassArgs A) {
-    pass_body<LAYOUT, N, C, WC, SV, TH>(in, out, A);
+    pass_body<LAYOUT, N, C, WC, true, SV, TH>(in, out, A);
 }
 
 }  // namespace croft

@@ -348,6 +348,8 @@ static croft_status add_axis_pass(croft_plan p, int axis, int x0 = 0, int nxs = 
     L.args.tw64 = f64 ? (const double2*)p->tw_dev[axis] : nullptr;
     L.args.tc_b = p->tc_b;
     L.args.status = p->d_status;
+    // y after z, both over the whole grid plane by plane: from the last plane to the first (col_tile)
+    L.args.backwards = (axis == 1 && layout == LAYOUT_COL && nxs < 0 && p->passes.size() == 1) ? 1 : 0;
     L.offset = offset;
     L.src_in = sin;
     L.group = grp;

@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(256, tc_two_minb(N)) croft_tc_two_kernel(const
         c = tid % W;
         lane = tid / W;
     }
-    const long long col = (long long)blockIdx.x * W + c;
+    const long long col = (LAYOUT == LAYOUT_ROW ? (long long)blockIdx.x : (long long)col_tile(A, blockIdx.x, gridDim.x)) * W + c;
     const bool ok = col < A.ncols;
     long long base = 0, M = 1;
     if constexpr (LAYOUT == LAYOUT_ROW) {

@@ -146,7 +146,7 @@ __global__ void __cluster_dims__(2, 1, 1)
     pdl_allow_dependents();
     pdl_wait();
     const int c = threadIdx.x % W, lane = threadIdx.x / W;
-    const long long col = (long long)(blockIdx.x / 2) * W + c;
+    const long long col = (long long)col_tile(A, blockIdx.x / 2, gridDim.x / 2) * W + c;
     const bool ok = col < A.ncols;
     long long b_, m_;
     col_split(col, A, b_, m_);
@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(croft_two_col(N, LONG).w* croft_two_col(N, LON
     const float2* tw = two_twiddles<N, K.stage != 0>(A.tw, two_smem, K.w * K.t);
     pdl_wait();
     const int c = threadIdx.x % K.w, lane = threadIdx.x / K.w;
-    const long long col = (long long)blockIdx.x * K.w + c;
+    const long long col = (long long)col_tile(A, blockIdx.x, gridDim.x) * K.w + c;
     const bool ok = col < A.ncols;
     long long b, m;
     col_split(col, A, b, m);
