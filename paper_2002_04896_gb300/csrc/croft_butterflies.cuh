@@ -32,7 +32,37 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
     return make_double2(fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x));
 }
 
+// complex64 whose sums and differences take one instruction for both parts (add and fma .f32x2 of sm_100 and later; the
+// same roundings as float2's).  Kernels that are bound by instruction issue or by the length of their
+// butterflies gain a few per cent, kernels short of registers lose to the pairing: each two-stage kernel
+// has the measured choice in its table (croft_two_stage.h).
+struct __align__(8) packed2 {
+    float x, y;
+};
+__device__ __forceinline__ packed2 cadd(packed2 a, packed2 b) {
+    packed2 r;
+    asm("{\n .reg .b64 p, q;\n mov.b64 p, {%2, %3};\n mov.b64 q, {%4, %5};\n add.rn.f32x2 p, p, q;\n mov.b64 {%0, %1}, p;\n}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+__device__ __forceinline__ packed2 csub(packed2 a, packed2 b) {
+    packed2 r;
+    asm("{\n .reg .b64 p, q, m;\n mov.b64 p, {%2, %3};\n mov.b64 q, {%4, %5};\n mov.b64 m, {%6, %6};\n fma.rn.f32x2 p, q, m, p;\n"
+        " mov.b64 {%0, %1}, p;\n}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(-1.f));
+    return r;
+}
+__device__ __forceinline__ packed2 cmul(packed2 a, packed2 b) {
+    packed2 r;
+    r.x = fmaf(a.x, b.x, -a.y * b.y);
+    r.y = fmaf(a.x, b.y, a.y * b.x);
+    return r;
+}
+
 template <class C> struct CxScalar;
+template <> struct CxScalar<packed2> { using T = float; };
 template <> struct CxScalar<float2> { using T = float; };
 template <> struct CxScalar<double2> { using T = double; };
 
@@ -84,8 +114,9 @@ template <class C> __device__ __forceinline__ void dft4(C& x0, C& x1, C& x2, C& 
     C c = cadd(x1, x3), d = mul_mi(csub(x1, x3));
     x0 = cadd(a, c);
     x2 = csub(a, c);
-    x1 = cadd(b, d);
-    x3 = csub(b, d);
+    // (rotated by -i: a swap of the parts, which a pair of scalar sums has for nothing)
+    x1 = mkc<C>(b.x + d.x, b.y + d.y);
+    x3 = mkc<C>(b.x - d.x, b.y - d.y);
 }
 
 template <int R, class C> struct Dft;

@@ -31,6 +31,7 @@ namespace croft {
 // Conjugates v when isign = -1.  (complex128: by the sign bit, on the integer pipe; a multiply by isign
 // at the load and at the store is 2 of the 23 instructions a point of a 128-point pass on the FP64 pipe.)
 __device__ __forceinline__ void conj_if(float2& v, float isign) { v.y *= isign; }
+__device__ __forceinline__ void conj_if(packed2& v, float isign) { v.y *= isign; }
 __device__ __forceinline__ void conj_if(double2& v, float isign) {
     const int flip = __float_as_int(isign) & 0x80000000;
     v.y = __hiloint2double(__double2hiint(v.y) ^ flip, __double2loint(v.y));

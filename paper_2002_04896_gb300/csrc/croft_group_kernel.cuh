@@ -55,10 +55,12 @@ template <int LAYOUT, int N>
 __global__ void __launch_bounds__(group_two<LAYOUT, N>().w* group_two<LAYOUT, N>().t, group_two<LAYOUT, N>().minb)
     croft_group_two_kernel(const __grid_constant__ GroupArgs A) {
     constexpr CroftTwo K = group_two<LAYOUT, N>();
-    extern __shared__ __align__(16) float2 two_smem[];
-    float2* buf = two_smem + (K.stage ? croft_two_pad(N) : 0);
+    using C = typename TwoComplex<K.packed != 0>::type;
+    extern __shared__ __align__(16) float2 two_raw[];
+    C* two_smem = reinterpret_cast<C*>(two_raw);
+    C* buf = two_smem + (K.stage ? croft_two_pad(N) : 0);
     pdl_allow_dependents();
-    const float2* tw = two_twiddles<N, K.stage != 0>(A.tw, two_smem, K.w * K.t);
+    const C* tw = two_twiddles<N, K.stage != 0>(A.tw, two_smem, K.w * K.t);
     const GroupSeg S = A.segs[A.cta_seg[blockIdx.x]];
     const long long tile = (long long)blockIdx.x - S.first_tile;
     pdl_wait();
@@ -66,14 +68,16 @@ __global__ void __launch_bounds__(group_two<LAYOUT, N>().w* group_two<LAYOUT, N>
         const int c = threadIdx.x / K.t, lane = threadIdx.x % K.t;
         const long long col = tile * K.w + c;
         const long long base = col * N;
-        two_pencil<N, K.r1, K.t>(GlobalInUnit{S.in + base, A.isign}, GlobalOutUnit{S.out + base, A.isign},
-                                 TwoExRow<K.r1, float2>{buf + c * K.ld}, tw, lane, col < S.ncols);
+        two_pencil<N, K.r1, K.t>(GlobalInUnitT<C>{reinterpret_cast<const C*>(S.in) + base, A.isign},
+                             GlobalOutUnitT<C>{reinterpret_cast<C*>(S.out) + base, A.isign},
+                                 TwoExRow<K.r1, C>{buf + c * K.ld}, tw, lane, col < S.ncols);
     } else {
         const int c = threadIdx.x % K.w, lane = threadIdx.x / K.w;
         const long long col = tile * K.w + c;
         const long long base = group_col_base(S, col, N);
-        two_pencil<N, K.r1, K.t>(GlobalIn{S.in + base, S.M, A.isign}, GlobalOut{S.out + base, S.M, A.isign},
-                                 TwoExCol<K.r1, K.w, float2>{buf + c}, tw, lane, col < S.ncols);
+        two_pencil<N, K.r1, K.t>(GlobalInT<C>{reinterpret_cast<const C*>(S.in) + base, S.M, A.isign},
+                             GlobalOutT<C>{reinterpret_cast<C*>(S.out) + base, S.M, A.isign},
+                                 TwoExCol<K.r1, K.w, C>{buf + c}, tw, lane, col < S.ncols);
     }
 }
 

@@ -231,18 +231,17 @@ static int rules_sv(croft_plan p, int axis) {
 // complex64 CUDA-core passes that the rules plan.  A tuned plan's choice and the measurement switches
 // CROFT_RING, CROFT_PAIR and CROFT_COL_TH name a kernel and keep it; CROFT_TWO_STAGE=0 switches the
 // two-stage kernels off.
-static croft_status attach_two(croft_plan p, int axis, PassLaunch& L) {
+static void attach_two(croft_plan p, int axis, PassLaunch& L) {
     memset(&L.two, 0, sizeof(L.two));
     const char* te = getenv("CROFT_TWO_STAGE");
     if (L.f64 || L.tc || p->axis_kind[axis] >= 0 || (te && te[0] == '0') || getenv("CROFT_RING") || getenv("CROFT_PAIR") ||
         getenv("CROFT_COL_TH"))
-        return CROFT_OK;
+        return;
     shape_two(L.two, L.layout, L.args.n, L.args.M, L.args.ncols);
-    if (!L.two.fn) return CROFT_OK;
+    if (!L.two.fn) return;
     const int n = L.args.n;
     L.two.tw = p->tw_dev[axis] + n;  // (the axis's second table)
     host_build_two_twiddles(n, L.two.r1, p->tw_host[axis].data() + 2 * (size_t)n);
-    return CROFT_OK;
 }
 
 static croft_status add_axis_pass(croft_plan p, int axis, int x0 = 0, int nxs = -1, int group = -1, int src_in = -1) {
@@ -290,9 +289,8 @@ static croft_status add_axis_pass(croft_plan p, int axis, int x0 = 0, int nxs = 
             L.offset = offset;
             L.src_in = sin;
             L.group = grp;
-            if (prepare_pass(L) == cudaSuccess) {
-                const croft_status st = attach_two(p, axis, L);
-                if (st != CROFT_OK) return st;
+            attach_two(p, axis, L);
+            if (L.two.fn || prepare_pass(L) == cudaSuccess) {
                 p->passes.push_back(L);
                 p->pass_axis.push_back(axis);
                 if (grp >= p->ngroups) p->ngroups = grp + 1;
@@ -353,9 +351,8 @@ static croft_status add_axis_pass(croft_plan p, int axis, int x0 = 0, int nxs = 
     L.offset = offset;
     L.src_in = sin;
     L.group = grp;
-    if (prepare_pass(L) != cudaSuccess) return CROFT_ERR_CUDA;
-    const croft_status ts = attach_two(p, axis, L);
-    if (ts != CROFT_OK) return ts;
+    attach_two(p, axis, L);
+    if (!L.two.fn && prepare_pass(L) != cudaSuccess) return CROFT_ERR_CUDA;
     p->passes.push_back(L);
     p->pass_axis.push_back(axis);
     if (grp >= p->ngroups) p->ngroups = grp + 1;
@@ -444,10 +441,17 @@ static croft_status add_plane_pass(croft_plan p, const PlaneKernel* pk) {
     return CROFT_OK;
 }
 
-// The complex64 tables of every axis, in one copy each.
+// The complex64 tables of every axis, in one copy each; an axis's own table only where a pass without a two-stage
+// kernel, or the general convolution kernel, reads it.
 static croft_status upload_tables(croft_plan p) {
     for (int a = 0; a < 3; ++a) {
         std::vector<float>& t = p->tw_host[a];
+        bool own = p->conv_fused && p->conv_axis == a && p->conv.args.tw == p->tw_dev[a];
+        for (size_t i = 0; i < p->passes.size(); ++i)
+            own = own || (p->pass_axis[i] == a && !p->passes[i].two.fn) || p->passes[i].kind == PASS_PLANE;
+        if (!t.empty() && own && p->tw_sched[a].count > 0 &&
+            build_twiddles(p->dims[a], p->tw_sched[a].r, p->tw_sched[a].count, t.data()) != p->dims[a] - 1)
+            return CROFT_ERR_CUDA;
         if (!t.empty() && cudaMemcpy(p->tw_dev[a], t.data(), sizeof(float) * t.size(), cudaMemcpyHostToDevice) != cudaSuccess)
             return CROFT_ERR_CUDA;
         std::vector<float>().swap(t);
@@ -473,7 +477,7 @@ static void plan_conv(croft_plan p) {
     const long long M = (axis == 2) ? 1 : (axis == 1 ? (long long)p->dims[2] : (long long)p->dims[1] * p->dims[2]);
     if (f64 ? !conv64_kernel_for(n) : !conv_kernel_for(n)) return;
     PassLaunch L;
-    const CroftTwo K = f64 ? CroftTwo{0, 0, 0, 0, 0, 0, 0} : croft_two_conv(n);
+    const CroftTwo K = f64 ? CroftTwo{0, 0, 0, 0, 0, 0, 0, 0} : croft_two_conv(n);
     if (K.r1) {  // two stages (croft_two_conv_kernel.cuh)
         memset(&L, 0, sizeof(L));
         const long long ncols = N / n, grid = (ncols + K.w - 1) / K.w;
@@ -639,8 +643,12 @@ static croft_status create_impl(croft_plan* out, int nx, int ny, int nz, croft_d
         }
         // (room for three more tables behind it: attach_two, plan_zy, plan_conv; upload_tables copies all four)
         p->tw_host[axis].assign(8 * (size_t)n, 0.f);
-        if (p->axis_tc[axis] && croft_tc_two(n)) host_build_two_twiddles(n, 16, p->tw_host[axis].data());
-        else if (build_twiddles(n, rad, ns, p->tw_host[axis].data()) != n - 1) return fail(p, CROFT_ERR_UNSUPPORTED_SIZE);
+        if (p->axis_tc[axis] && croft_tc_two(n)) {
+            host_build_two_twiddles(n, 16, p->tw_host[axis].data());
+        } else {  // (the first table itself only where a kernel reads it: upload_tables)
+            p->tw_sched[axis].count = ns;
+            for (int i = 0; i < ns; ++i) p->tw_sched[axis].r[i] = rad[i];
+        }
         if (dev_alloc((void**)&p->tw_dev[axis], sizeof(float2) * 4 * (size_t)n) != cudaSuccess) return fail(p, CROFT_ERR_OOM);
     }
 

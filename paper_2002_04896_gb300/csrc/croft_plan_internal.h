@@ -25,6 +25,7 @@ struct croft_plan_s {
     float2* tw_dev[3];                // per-axis twiddle tables (NULL for length <= 1): the pass's own, then
                                       // (complex64) n entries each for its two-stage kernel, the plane
                                       // pass and the fused convolution
+    CroftSched tw_sched[3];           // complex64: the schedule of the axis's own table (count 0: none or built already)
     std::vector<float> tw_host[3];    // complex64 tables until their upload at the end of creation
     croft::PlanePass zy;              // z and y in one pass over the planes (fn NULL: axis by axis)
     float2* tw_pair[3];               // pair column passes: [half-length table | combine twiddles], else NULL

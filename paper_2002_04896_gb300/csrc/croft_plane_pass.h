@@ -43,16 +43,18 @@ CROFT_HD constexpr int croft_plane_smem(int ny, int nz) { return ny * croft_plan
 // 96^3 0.94, 100^3 1.14, 108^3 0.89; 300 planes of 48^2 1.41, 54^2 1.48, 60^2 1.40, 64^2 1.25, 80^2 1.08, 90^2
 // 1.20, 96^2 1.13, 100^2 1.05, 108^2 1.00, 120^2 0.96; 4 planes of 64^2 0.92, 16 of 96^2 0.69.  Launched one by
 // one, a transform of up to about 64^3 points takes as long as its launches (9 us for three, 5 for two), so
-// planes of up to 4096 points always take it; larger ones up to 10,000 from about two planes per SM on (162 of
-// 90 x 108, one round and a rest: a convolution takes 36.6 us against 35.3).
+// planes of up to 4096 points always take it; larger ones from about two planes per SM on (162 of 90 x 108, one
+// round and a rest: a convolution takes 36.6 us against 35.3), up to 6400 points, and up to 10,000 while the grid
+// stays in the L2 (z and y of 960 planes, two passes / plane pass: 72^2 30.4 / 27.4 us, 80^2 35.3 / 35.8, 96^2
+// 48.4 / 54.0, 108^2 60 / 67).
 CROFT_HD constexpr bool croft_plane_pass_rule(int nx, int ny, int nz) {
     return croft_plane_r1(ny) != 0 && croft_plane_r1(nz) != 0 &&
-           (ny * nz <= 4096 || (ny * nz <= 10000 && nx >= 288));
+           (ny * nz <= 4096 || (nx >= 288 && (ny * nz <= 6400 || (ny * nz <= 10000 && nx <= 456))));
 }
 // Threads of a plane's CTA: enough for one round of butterflies a stage where an SM holds one plane, fewer (and
 // more planes at a time) where there are many.  64^3: 128 / 256 / 384 / 512 / 1024 threads 0.81 / 0.89 / 0.88 /
 // 0.92 / 0.90 of the three passes' speed, 300 planes of 64^2 1.12 / 1.25 / 1.02 / 1.02 / 0.91, 4096 of 32^2
-// 1.20 / 1.15 / 1.04 / 1.05 / 0.79.
+// 1.20 / 1.15 / 1.04 / 1.05 / 0.79; 960 planes of 60^2 27.0 / 23.9 / 25.6 / 26.3 / 31.2 us.
 CROFT_HD constexpr int croft_plane_threads(int nx, int ny, int nz) {
-    return nx <= 152 ? 512 : (nx <= 608 ? 256 : (ny * nz <= 1600 ? 128 : 192));
+    return nx <= 152 ? 512 : (nx <= 608 || ny * nz > 1600 ? 256 : 128);
 }

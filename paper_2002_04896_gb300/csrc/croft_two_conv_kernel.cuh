@@ -22,15 +22,16 @@
 namespace croft {
 
 // Shared memory: [twiddles when STAGE][tile: N x W complex][G tile: N x W real].
-template <int N, int R1, int T, int W, bool STAGE>
-__device__ __forceinline__ void two_conv_body(const float2* in, float2* out, const float* g, const PassArgs& A) {
+template <int N, int R1, int T, int W, bool STAGE, class C>
+__device__ __forceinline__ void two_conv_body(const C* in, C* out, const float* g, const PassArgs& A) {
     constexpr int R2 = N / R1;
     constexpr int Q1 = (R2 + T - 1) / T, Q2 = (R1 + T - 1) / T;
-    extern __shared__ __align__(16) float2 two_smem[];
-    float2* tile = two_smem + (STAGE ? croft_two_pad(N) : 0);
+    extern __shared__ __align__(16) float2 two_raw[];
+    C* two_smem = reinterpret_cast<C*>(two_raw);
+    C* tile = two_smem + (STAGE ? croft_two_pad(N) : 0);
     const int c = threadIdx.x % W, lane = threadIdx.x / W;
     float* gs = reinterpret_cast<float*>(tile + N * W) + c;
-    const TwoExCol<R1, W, float2> ex{tile + c};
+    const TwoExCol<R1, W, C> ex{tile + c};
     const long long col = (long long)blockIdx.x * W + c;
     const bool ok = col < A.ncols;
     long long b_, m_;
@@ -48,12 +49,12 @@ __device__ __forceinline__ void two_conv_body(const float2* in, float2* out, con
         }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
-    const float2* tw = two_twiddles<N, STAGE>(A.tw, two_smem, W * T);
+    const C* tw = two_twiddles<N, STAGE>(A.tw, two_smem, W * T);
     pdl_wait();  // (G and the twiddles are not written by the previous pass)
 
     {
-        const GlobalIn src{in + base, A.M, 1.f};
-        float2 v[Q1][R1];
+        const GlobalInT<C> src{in + base, A.M, 1.f};
+        C v[Q1][R1];
 #pragma unroll
         for (int q = 0; q < Q1; ++q) {
             const int b = lane + q * T;
@@ -78,7 +79,7 @@ __device__ __forceinline__ void two_conv_body(const float2* in, float2* out, con
     for (int q = 0; q < Q2; ++q) {
         const int k = lane + q * T;
         if (R1 % T == 0 || k < R1) {
-            float2 v[R2];
+            C v[R2];
 #pragma unroll
             for (int j = 0; j < R2; ++j) v[j] = *ex.at(j, k);
 #pragma unroll
@@ -87,7 +88,7 @@ __device__ __forceinline__ void two_conv_body(const float2* in, float2* out, con
 #pragma unroll
             for (int j = 0; j < R2; ++j) {
                 const float ga = gs[(k + j * R1) * W];
-                v[j] = make_float2(v[j].x * ga, -(v[j].y * ga));
+                v[j] = mkc<C>(v[j].x * ga, -(v[j].y * ga));
             }
             dft<R2>(v);
 #pragma unroll
@@ -95,12 +96,12 @@ __device__ __forceinline__ void two_conv_body(const float2* in, float2* out, con
         }
     }
     __syncthreads();
-    const GlobalOut dst{out + base, A.M, -1.f};
+    const GlobalOutT<C> dst{out + base, A.M, -1.f};
 #pragma unroll
     for (int q = 0; q < Q1; ++q) {
         const int b = lane + q * T;
         if (R2 % T == 0 || b < R2) {
-            float2 v[R1];
+            C v[R1];
 #pragma unroll
             for (int j = 0; j < R1; ++j) v[j] = *ex.at(b, j);
 #pragma unroll
@@ -118,7 +119,8 @@ template <int N>
 __global__ void __launch_bounds__(croft_two_conv(N).w* croft_two_conv(N).t, croft_two_conv(N).minb)
     croft_two_conv_kernel(const float2* in, float2* out, const float* g, const __grid_constant__ PassArgs A) {
     constexpr CroftTwo K = croft_two_conv(N);
-    two_conv_body<N, K.r1, K.t, K.w, K.stage != 0>(in, out, g, A);
+    using C = typename TwoComplex<K.packed != 0>::type;
+    two_conv_body<N, K.r1, K.t, K.w, K.stage != 0>(reinterpret_cast<const C*>(in), reinterpret_cast<C*>(out), g, A);
 }
 
 }  // namespace croft

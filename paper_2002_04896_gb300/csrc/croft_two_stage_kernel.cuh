@@ -111,9 +111,14 @@ struct TwoExRow {
     __device__ __forceinline__ C* at(int b, int j) const { return s + b * (R1 + D) + j; }
 };
 
+// The complex type of a kernel's arithmetic (packed2: paired sums).
+template <bool PACKED> struct TwoComplex { using type = float2; };
+template <> struct TwoComplex<true> { using type = packed2; };
+
 // Twiddles: staged (copied to `stw`, which the barrier between the stages publishes) or as they are.
-template <int N, bool STAGE>
-__device__ __forceinline__ const float2* two_twiddles(const float2* tw, float2* stw, int threads) {
+template <int N, bool STAGE, class C>
+__device__ __forceinline__ const C* two_twiddles(const float2* twg, C* stw, int threads) {
+    const C* tw = reinterpret_cast<const C*>(twg);
     if constexpr (STAGE) {
         for (int i = threadIdx.x; i < N; i += threads) stw[i] = tw[i];
         return stw;
@@ -139,7 +144,9 @@ __global__ void __cluster_dims__(2, 1, 1)
     constexpr int H1 = (R2 + 1) / 2, H2 = (R1 + 1) / 2;  // butterflies of CTA 0 in the two stages
     constexpr int Q1 = (H1 + T - 1) / T, Q2 = (H2 + T - 1) / T;
     namespace cg = cooperative_groups;
-    extern __shared__ __align__(16) float2 two_smem[];
+    using C = typename TwoComplex<K.packed != 0>::type;
+    extern __shared__ __align__(16) float2 two_raw[];
+    C* two_smem = reinterpret_cast<C*>(two_raw);
     const cg::cluster_group cluster = cg::this_cluster();
     const int r = (int)cluster.block_rank();
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
@@ -152,8 +159,8 @@ __global__ void __cluster_dims__(2, 1, 1)
     col_split(col, A, b_, m_);
     const long long base = b_ * (long long)N * A.M + m_;
     {
-        const GlobalIn src{in + base, A.M, A.isign};
-        float2 v[Q1][R1];
+        const GlobalInT<C> src{reinterpret_cast<const C*>(in) + base, A.M, A.isign};
+        C v[Q1][R1];
 #pragma unroll
         for (int q = 0; q < Q1; ++q) {
             const int lb = lane + q * T, b = r * H1 + lb;
@@ -165,8 +172,8 @@ __global__ void __cluster_dims__(2, 1, 1)
 #pragma unroll
         for (int q = 0; q < Q1; ++q) dft<R1>(v[q]);
         asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
-        float2* first = (r == 0 ? two_smem : cluster.map_shared_rank(two_smem, 0)) + c;
-        float2* second = (r == 1 ? two_smem : cluster.map_shared_rank(two_smem, 1)) + c;
+        C* first = (r == 0 ? two_smem : cluster.map_shared_rank(two_smem, 0)) + c;
+        C* second = (r == 1 ? two_smem : cluster.map_shared_rank(two_smem, 1)) + c;
 #pragma unroll
         for (int q = 0; q < Q1; ++q) {
             const int lb = lane + q * T, b = r * H1 + lb;
@@ -177,16 +184,17 @@ __global__ void __cluster_dims__(2, 1, 1)
         }
     }
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-    const GlobalOut dst{out + base, A.M, A.isign};
+    const GlobalOutT<C> dst{reinterpret_cast<C*>(out) + base, A.M, A.isign};
+    const C* tw = reinterpret_cast<const C*>(A.tw);
 #pragma unroll
     for (int q = 0; q < Q2; ++q) {
         const int lk = lane + q * T, k = r * H2 + lk;
         if (lk < H2 && k < R1) {
-            float2 v[R2];
+            C v[R2];
 #pragma unroll
             for (int j = 0; j < R2; ++j) v[j] = two_smem[(j * H2 + lk) * W + c];
 #pragma unroll
-            for (int j = 1; j < R2; ++j) v[j] = cmul(v[j], A.tw[j * R1 + k]);
+            for (int j = 1; j < R2; ++j) v[j] = cmul(v[j], tw[j * R1 + k]);
             dft<R2>(v);
             if (ok) {
 #pragma unroll
@@ -202,10 +210,12 @@ template <int N, bool LONG>
 __global__ void __launch_bounds__(croft_two_col(N, LONG).w* croft_two_col(N, LONG).t, croft_two_col(N, LONG).minb)
     croft_two_col_kernel(const float2* in, float2* out, const __grid_constant__ PassArgs A) {
     constexpr CroftTwo K = croft_two_col(N, LONG);
-    extern __shared__ __align__(16) float2 two_smem[];
-    float2* tile = two_smem + (K.stage ? croft_two_pad(N) : 0);
+    using C = typename TwoComplex<K.packed != 0>::type;
+    extern __shared__ __align__(16) float2 two_raw[];
+    C* two_smem = reinterpret_cast<C*>(two_raw);
+    C* tile = two_smem + (K.stage ? croft_two_pad(N) : 0);
     pdl_allow_dependents();
-    const float2* tw = two_twiddles<N, K.stage != 0>(A.tw, two_smem, K.w * K.t);
+    const C* tw = two_twiddles<N, K.stage != 0>(A.tw, two_smem, K.w * K.t);
     pdl_wait();
     const int c = threadIdx.x % K.w, lane = threadIdx.x / K.w;
     const long long col = (long long)col_tile(A, blockIdx.x, gridDim.x) * K.w + c;
@@ -213,8 +223,9 @@ __global__ void __launch_bounds__(croft_two_col(N, LONG).w* croft_two_col(N, LON
     long long b, m;
     col_split(col, A, b, m);
     const long long base = b * (long long)N * A.M + m;
-    two_pencil<N, K.r1, K.t>(GlobalIn{in + base, A.M, A.isign}, GlobalOut{out + base, A.M, A.isign},
-                             TwoExCol<K.r1, K.w, float2>{tile + c}, tw, lane, ok);
+    two_pencil<N, K.r1, K.t>(GlobalInT<C>{reinterpret_cast<const C*>(in) + base, A.M, A.isign},
+                             GlobalOutT<C>{reinterpret_cast<C*>(out) + base, A.M, A.isign},
+                             TwoExCol<K.r1, K.w, C>{tile + c}, tw, lane, ok);
 }
 
 // The row pass: W contiguous pencils per CTA, T threads per pencil.
@@ -222,17 +233,20 @@ template <int N>
 __global__ void __launch_bounds__(croft_two_row(N).w* croft_two_row(N).t, croft_two_row(N).minb)
     croft_two_row_kernel(const float2* in, float2* out, const __grid_constant__ PassArgs A) {
     constexpr CroftTwo K = croft_two_row(N);
-    extern __shared__ __align__(16) float2 two_smem[];
-    float2* tile = two_smem + (K.stage ? croft_two_pad(N) : 0);
+    using C = typename TwoComplex<K.packed != 0>::type;
+    extern __shared__ __align__(16) float2 two_raw[];
+    C* two_smem = reinterpret_cast<C*>(two_raw);
+    C* tile = two_smem + (K.stage ? croft_two_pad(N) : 0);
     pdl_allow_dependents();
-    const float2* tw = two_twiddles<N, K.stage != 0>(A.tw, two_smem, K.w * K.t);
+    const C* tw = two_twiddles<N, K.stage != 0>(A.tw, two_smem, K.w * K.t);
     pdl_wait();
     const int c = threadIdx.x / K.t, lane = threadIdx.x % K.t;
     const long long col = (long long)blockIdx.x * K.w + c;
     const bool ok = col < A.ncols;
     const long long base = col * N;
-    two_pencil<N, K.r1, K.t>(GlobalInUnit{in + base, A.isign}, GlobalOutUnit{out + base, A.isign},
-                             TwoExRow<K.r1, float2>{tile + c * K.ld}, tw, lane, ok);
+    two_pencil<N, K.r1, K.t>(GlobalInUnitT<C>{reinterpret_cast<const C*>(in) + base, A.isign},
+                             GlobalOutUnitT<C>{reinterpret_cast<C*>(out) + base, A.isign},
+                             TwoExRow<K.r1, C>{tile + c * K.ld}, tw, lane, ok);
 }
 
 }  // namespace croft
