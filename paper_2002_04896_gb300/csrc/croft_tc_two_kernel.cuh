@@ -10,7 +10,7 @@
 //
 // What bounds it: the latency of that chain at three or four 256-thread CTAs per SM (five barriers and an MMA round trip
 // in it); the tensor pipe idles.  Against three stages (16, then the near-equal split of the rest: one exchange and
-// two barriers more, at 32 threads per pencil) a 512^3 bf16x3 forward transform went from 1630 to 1394 us, 256^3 from 184 to 152.
+// two barriers more, at 32 threads per pencil) a 512^3 bf16x3 forward transform went from 1630 to 1364 us, 256^3 from 184 to 149.
 // The next pass may become resident while this one drains (programmatic dependent launch): all of this
 // launch's CTAs run by then, so a waiting CTA's TMEM allocation delays none of them.
 #pragma once
@@ -34,6 +34,13 @@ CROFT_HD constexpr int tc_two_smem(int n, bool row) {
 // 256^3 with three / four 169 / 152.
 CROFT_HD constexpr int tc_two_minb(int n) { return n / 16 <= 16 ? 4 : 3; }
 
+// Paired sums (packed2) in the second stage: where they measured faster (x or z pass, us: 384 points 254 -> 250, 432 205 ->
+// 197, 288 213 -> 209, 512 499 -> 487; 320 246 -> 257 the other way, the rest equal).
+CROFT_HD constexpr bool tc_two_packed(int n) { return n == 288 || n == 384 || n == 432 || n == 512; }
+
+// The y pass follows A.backwards (256^3 53.2 -> 51.2 us, 400 points 194.7 -> 190.5), but at 512 points, whose
+// registers are spent: 469 -> 485 us with the choice of the tile compiled in.
+//
 // Shared memory: [B operand: 4 KB][A operands: Q x 256 rows of 128 bytes | exchange buffer].
 template <int LAYOUT, int N, int PREC>
 __global__ void __launch_bounds__(256, tc_two_minb(N)) croft_tc_two_kernel(const float2* in, float2* out,
@@ -65,7 +72,7 @@ __global__ void __launch_bounds__(256, tc_two_minb(N)) croft_tc_two_kernel(const
         c = tid % W;
         lane = tid / W;
     }
-    const long long col = (LAYOUT == LAYOUT_ROW ? (long long)blockIdx.x : (long long)col_tile(A, blockIdx.x, gridDim.x)) * W + c;
+    const long long col = (long long)(LAYOUT == LAYOUT_COL && N < 512 ? col_tile(A, blockIdx.x, gridDim.x) : blockIdx.x) * W + c;
     const bool ok = col < A.ncols;
     long long base = 0, M = 1;
     if constexpr (LAYOUT == LAYOUT_ROW) {
@@ -165,21 +172,24 @@ __global__ void __launch_bounds__(256, tc_two_minb(N)) croft_tc_two_kernel(const
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     if (tid < 32) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(NCOLS));
+    using C = typename TwoComplex<tc_two_packed(N)>::type;
+    const C* tw = reinterpret_cast<const C*>(A.tw);
+    C* dst = reinterpret_cast<C*>(out) + base;
 #pragma unroll
     for (int q = 0; q < Q2; ++q) {
         const int k = lane + q * T;
-        float2 v[R2];
+        C v[R2];
 #pragma unroll
-        for (int j = 0; j < R2; ++j) v[j] = *at(j, k);
+        for (int j = 0; j < R2; ++j) v[j] = *reinterpret_cast<const C*>(at(j, k));
 #pragma unroll
-        for (int j = 1; j < R2; ++j) v[j] = cmul(v[j], A.tw[j * 16 + k]);
+        for (int j = 1; j < R2; ++j) v[j] = cmul(v[j], tw[j * 16 + k]);
         dft<R2>(v);
         if (ok) {
 #pragma unroll
             for (int j = 0; j < R2; ++j) {
                 conj_if(v[j], A.isign);
                 const int a = k + j * 16;
-                out[base + (LAYOUT == LAYOUT_ROW ? a : (long long)a * M)] = v[j];
+                dst[LAYOUT == LAYOUT_ROW ? a : (long long)a * M] = v[j];
             }
         }
     }
