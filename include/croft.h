@@ -198,9 +198,10 @@ croft_status croft_plan_create_batched_mode(croft_plan* out, int count, const in
  * croft_exec_batched_forward / _backward: in and out are HOST arrays of
  * `count` DEVICE pointers (grid g reads in[g], writes out[g]); each pair obeys
  * the single-grid rules (16-byte aligned, in[g] == out[g] or disjoint).
- * Stream-ordered.  The grids' descriptors travel through pinned host memory
- * owned by the plan, so an exec first waits (on the host) until the previous
- * exec of the same plan has started executing on the device.
+ * Stream-ordered.  ONE_LAUNCH and PER_PASS send the grids' descriptors through
+ * pinned host memory owned by the plan, so an exec of theirs first waits (on the
+ * host) until the previous exec of the same plan has started executing on the
+ * device; GROUPED passes them as kernel parameters and does not wait.
  * Device-side waits that run out set the plan's device status to
  * CROFT_ERR_TIMEOUT (croft_plan_last_device_status); the exec itself still
  * returns CROFT_OK in that case because it does not synchronise.

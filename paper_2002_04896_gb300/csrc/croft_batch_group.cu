@@ -7,6 +7,7 @@
 // kernel) reused for every pencil of that length, across grids as well.
 #include <cuda_runtime.h>
 
+#include <limits.h>
 #include <string.h>
 
 #include <algorithm>
@@ -43,28 +44,22 @@ void host_build_two_twiddles(int n, int r1, float* out);
 
 struct GroupLaunch {
     int pass, layout, n;
-    int seg_begin, nseg;  // segments [seg_begin, seg_begin + nseg) of the segment table
-    int cta_begin, ctas;  // entries of the CTA map
+    int nseg, ctas;
+    int grid_of[kGroupSegs];     // batch index of each segment
+    int reads_in[kGroupSegs];    // 1: the segment's pass is its grid's first pass (reads `in`)
+    GroupArgs args;              // (pointers and isign filled per exec)
+    cudaGraphNode_t node[2];     // its node in the graph of each direction
     int W, block, smem;
     int tw_off;           // float2 offset of N's twiddles in the pool
 };
 
 struct GroupState {
     std::vector<GroupLaunch> launches;
-    std::vector<int> seg_grid;   // batch index of each segment
-    std::vector<int> seg_first;  // 1: the segment's pass is its grid's first pass (reads `in`)
-    GroupSeg* staging = nullptr; // pinned, pointers filled per exec
-    GroupSeg* d_segs = nullptr;
-    unsigned short* d_cta = nullptr;
     float2* d_tw = nullptr;
-    int nseg = 0;
 };
 
 void group_state_destroy(GroupState* s) {
     if (!s) return;
-    if (s->staging) host_free(s->staging);
-    dev_free(s->d_segs);
-    dev_free(s->d_cta);
     dev_free(s->d_tw);
     delete s;
 }
@@ -75,8 +70,6 @@ croft_status group_state_build(const std::vector<int>& dims, const std::vector<i
     GroupState* s = new (std::nothrow) GroupState();
     if (!s) return CROFT_ERR_OOM;
     static const int kAxis[3] = {2, 1, 0};
-    std::vector<GroupSeg> segs;
-    std::vector<unsigned short> cta;
     std::vector<float> pool;
     std::map<std::pair<int, int>, int> tw_off;  // (length, first radix of a two-stage pass or 0) -> offset
     // first pass of each grid (lowest pass index whose axis is longer than 1)
@@ -132,105 +125,109 @@ croft_status group_state_build(const std::vector<int>& dims, const std::vector<i
                 L.smem = (int)((tw_pad + tile_elems) * sizeof(float2));
             }
             L.tw_off = tw_off[key];
-            L.seg_begin = (int)segs.size();
-            L.cta_begin = (int)cta.size();
-            for (int i : kv.second) {
-                const int g = pgrid[i];
-                const long long N = (long long)dims[3 * g] * dims[3 * g + 1] * dims[3 * g + 2];
-                GroupSeg S;
-                memset(&S, 0, sizeof(S));
-                const int nz = dims[3 * g + 2], ny = dims[3 * g + 1];
-                S.M = kAxis[p] == 2 ? 1 : (kAxis[p] == 1 ? (long long)nz : (long long)ny * nz);
-                S.ncols = N / n;
-                S.cdiv = croft_coldiv_make(S.M, S.ncols + L.W);
-                S.first_tile = (int)(cta.size() - L.cta_begin);
-                const long long tiles = (S.ncols + L.W - 1) / L.W;
-                const int seg_local = (int)segs.size() - L.seg_begin;
-                if (seg_local > 65535 || (long long)cta.size() - L.cta_begin + tiles > 0x7fffffffLL) {
-                    group_state_destroy(s);
-                    return CROFT_ERR_UNSUPPORTED_SIZE;
-                }
-                for (long long t = 0; t < tiles; ++t) cta.push_back((unsigned short)seg_local);
-                segs.push_back(S);
-                s->seg_grid.push_back(g);
-                s->seg_first.push_back(first[i] == p ? 1 : 0);
-            }
-            L.nseg = (int)segs.size() - L.seg_begin;
-            L.ctas = (int)cta.size() - L.cta_begin;
+            L.nseg = L.ctas = 0;
+            memset(&L.args, 0, sizeof(L.args));
+            for (int& t : L.args.first_tile) t = INT_MAX;
             if (L.smem > 48 * 1024 && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, L.smem) != cudaSuccess) {
                 cudaGetLastError();
                 group_state_destroy(s);
                 return CROFT_ERR_CUDA;
             }
+            for (int i : kv.second) {
+                const int g = pgrid[i];
+                const long long N = (long long)dims[3 * g] * dims[3 * g + 1] * dims[3 * g + 2];
+                const int nz = dims[3 * g + 2], ny = dims[3 * g + 1];
+                if (L.nseg == kGroupSegs) {  // full: the rest in another launch
+                    s->launches.push_back(L);
+                    L.nseg = L.ctas = 0;
+                    for (int& t : L.args.first_tile) t = INT_MAX;
+                }
+                GroupSeg& S = L.args.seg[L.nseg];
+                S.M = kAxis[p] == 2 ? 1 : (kAxis[p] == 1 ? (long long)nz : (long long)ny * nz);
+                S.ncols = N / n;
+                S.cdiv = croft_coldiv_make(S.M, S.ncols + L.W);
+                const long long tiles = (S.ncols + L.W - 1) / L.W;
+                if (L.ctas + tiles > 0x7ffffffeLL) {
+                    group_state_destroy(s);
+                    return CROFT_ERR_UNSUPPORTED_SIZE;
+                }
+                L.args.first_tile[L.nseg] = L.ctas;
+                L.grid_of[L.nseg] = g;
+                L.reads_in[L.nseg] = first[i] == p ? 1 : 0;
+                L.ctas += (int)tiles;
+                ++L.nseg;
+            }
             s->launches.push_back(L);
         }
     }
-    s->nseg = (int)segs.size();
-    if (s->nseg == 0) {
+    if (s->launches.empty()) {
         *out = s;
         return CROFT_OK;
     }
-    if (host_alloc((void**)&s->staging, sizeof(GroupSeg) * s->nseg) != cudaSuccess ||
-        dev_alloc((void**)&s->d_segs, sizeof(GroupSeg) * s->nseg) != cudaSuccess ||
-        dev_alloc((void**)&s->d_cta, sizeof(unsigned short) * std::max<size_t>(1, cta.size())) != cudaSuccess ||
-        dev_alloc((void**)&s->d_tw, sizeof(float) * std::max<size_t>(2, pool.size())) != cudaSuccess) {
+    if (dev_alloc((void**)&s->d_tw, sizeof(float) * std::max<size_t>(2, pool.size())) != cudaSuccess) {
         cudaGetLastError();
         group_state_destroy(s);
         return CROFT_ERR_OOM;
     }
-    memcpy(s->staging, segs.data(), sizeof(GroupSeg) * s->nseg);
-    if (cudaMemcpy(s->d_cta, cta.data(), sizeof(unsigned short) * cta.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
-        (!pool.empty() && cudaMemcpy(s->d_tw, pool.data(), sizeof(float) * pool.size(), cudaMemcpyHostToDevice) != cudaSuccess)) {
+    if (!pool.empty() && cudaMemcpy(s->d_tw, pool.data(), sizeof(float) * pool.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
         cudaGetLastError();
         group_state_destroy(s);
         return CROFT_ERR_CUDA;
+    }
+    for (GroupLaunch& L : s->launches) {
+        L.args.tw = s->d_tw + L.tw_off;
+        L.args.W = L.W;
     }
     *out = s;
     return CROFT_OK;
 }
 
-// The grids' pointers for one exec (into the pinned staging table the graph uploads).
-void group_state_fill(GroupState* s, void* const* in, void* const* out) {
-    for (int k = 0; k < s->nseg; ++k) {
-        const int g = s->seg_grid[k];
-        s->staging[k].in = (const float2*)(s->seg_first[k] ? in[g] : out[g]);
-        s->staging[k].out = (float2*)out[g];
-    }
+static cudaKernelNodeParams group_node_params(const GroupLaunch& L, void** params) {
+    cudaKernelNodeParams kp;
+    memset(&kp, 0, sizeof(kp));
+    kp.func = (void*)group_kernel_for(L.layout, L.n);
+    kp.gridDim = dim3((unsigned)L.ctas, 1, 1);
+    kp.blockDim = dim3((unsigned)L.block, 1, 1);
+    kp.sharedMemBytes = (unsigned)L.smem;
+    kp.kernelParams = params;
+    return kp;
 }
 
-// Adds [segment upload] -> pass 0 launches -> pass 1 launches -> pass 2 launches to g.
+// The grids' pointers for the next launch of direction dir's graph: every kernel's parameters (a change
+// reaches later launches only, so an exec in flight keeps its own).
+croft_status group_graph_fill(GroupState* s, cudaGraphExec_t ge, int dir, void* const* in, void* const* out) {
+    for (GroupLaunch& L : s->launches) {
+        for (int k = 0; k < L.nseg; ++k) {
+            const int g = L.grid_of[k];
+            L.args.seg[k].in = (const float2*)(L.reads_in[k] ? in[g] : out[g]);
+            L.args.seg[k].out = (float2*)out[g];
+        }
+        L.args.isign = dir == 0 ? 1.f : -1.f;
+        void* params[1] = {&L.args};
+        const cudaKernelNodeParams kp = group_node_params(L, params);
+        if (cudaGraphExecKernelNodeSetParams(ge, L.node[dir], &kp) != cudaSuccess) {
+            cudaGetLastError();
+            return CROFT_ERR_CUDA;
+        }
+    }
+    return CROFT_OK;
+}
+
+// Adds pass 0 launches -> pass 1 launches -> pass 2 launches to direction dir's graph.
 // With pdl, the edges from one pass's launches to the next pass's are programmatic:
 // the next pass's CTAs may become resident (and load their twiddles) while the
 // previous pass drains, and wait in the kernel (griddepcontrol.wait) for every
 // upstream launch to complete before they read the grid.
-croft_status group_graph_add(GroupState* s, cudaGraph_t g, float isign, bool pdl) {
-    if (s->nseg == 0) return CROFT_OK;
-    cudaGraphNode_t up;
-    if (cudaGraphAddMemcpyNode1D(&up, g, nullptr, 0, s->d_segs, s->staging, sizeof(GroupSeg) * s->nseg,
-                                 cudaMemcpyHostToDevice) != cudaSuccess)
-        return CROFT_ERR_CUDA;
-    std::vector<cudaGraphNode_t> prev = {up};
+croft_status group_graph_add(GroupState* s, cudaGraph_t g, int dir, bool pdl) {
+    std::vector<cudaGraphNode_t> prev;
     for (int p = 0; p < 3; ++p) {
         std::vector<cudaGraphNode_t> cur;
-        for (const GroupLaunch& L : s->launches) {
+        for (GroupLaunch& L : s->launches) {
             if (L.pass != p) continue;
-            GroupArgs A;
-            memset(&A, 0, sizeof(A));
-            A.segs = s->d_segs + L.seg_begin;
-            A.cta_seg = s->d_cta + L.cta_begin;
-            A.tw = s->d_tw + L.tw_off;
-            A.W = L.W;
-            A.isign = isign;
-            void* params[1] = {&A};
-            cudaKernelNodeParams kp;
-            memset(&kp, 0, sizeof(kp));
-            kp.func = (void*)group_kernel_for(L.layout, L.n);
-            kp.gridDim = dim3((unsigned)L.ctas, 1, 1);
-            kp.blockDim = dim3((unsigned)L.block, 1, 1);
-            kp.sharedMemBytes = (unsigned)L.smem;
-            kp.kernelParams = params;
+            void* params[1] = {&L.args};
+            const cudaKernelNodeParams kp = group_node_params(L, params);
             cudaGraphNode_t kn;
-            if (p == 0 || !pdl) {
+            if (prev.empty() || !pdl) {
                 if (cudaGraphAddKernelNode(&kn, g, prev.data(), prev.size(), &kp) != cudaSuccess) return CROFT_ERR_CUDA;
             } else {
                 if (cudaGraphAddKernelNode(&kn, g, nullptr, 0, &kp) != cudaSuccess) return CROFT_ERR_CUDA;
@@ -247,6 +244,7 @@ croft_status group_graph_add(GroupState* s, cudaGraph_t g, float isign, bool pdl
                         return CROFT_ERR_CUDA;
                 }
             }
+            L.node[dir] = kn;
             cur.push_back(kn);
         }
         if (!cur.empty()) prev = cur;

@@ -48,8 +48,8 @@ int host_build_twiddles(int n, float* out);  // croft_plan.cu
 struct GroupState;  // croft_batch_group.cu
 croft_status group_state_build(const std::vector<int>& dims, const std::vector<int>& pgrid, GroupState** out);
 void group_state_destroy(GroupState* s);
-void group_state_fill(GroupState* s, void* const* in, void* const* out);
-croft_status group_graph_add(GroupState* s, cudaGraph_t g, float isign, bool pdl);
+croft_status group_graph_fill(GroupState* s, cudaGraphExec_t ge, int dir, void* const* in, void* const* out);
+croft_status group_graph_add(GroupState* s, cudaGraph_t g, int dir, bool pdl);
 int group_state_launches(const GroupState* s);
 
 struct BatchState {
@@ -238,7 +238,7 @@ static croft_status build_graphs(BatchState* b) {
         b->graph[d] = g;
         if (b->mode == CROFT_BATCH_GROUPED) {
             const char* pdl_env = getenv("CROFT_PDL");  // 0: ordinary graph edges between the passes
-            croft_status st = group_graph_add(b->group, g, isign, !(pdl_env && pdl_env[0] == '0'));
+            croft_status st = group_graph_add(b->group, g, d, !(pdl_env && pdl_env[0] == '0'));
             if (st != CROFT_OK) return st;
             if (cudaGraphInstantiate(&b->gexec[d], g, 0) != cudaSuccess) return CROFT_ERR_CUDA;
             continue;
@@ -302,12 +302,14 @@ static croft_status exec_batch(croft_plan plan, void* const* in, void* const* ou
     const bool tm = plan->timing;
     if (tm && cudaEventRecord(plan->ev[0], s) != cudaSuccess) { cudaGetLastError(); return CROFT_ERR_CUDA; }
     if (b->gexec[dir]) {
-        if (b->staging_pending && cudaEventSynchronize(b->staging_free) != cudaSuccess) {
+        const bool grouped = b->mode == CROFT_BATCH_GROUPED;
+        if (!grouped && b->staging_pending && cudaEventSynchronize(b->staging_free) != cudaSuccess) {
             cudaGetLastError();
             return CROFT_ERR_CUDA;
         }
-        if (b->mode == CROFT_BATCH_GROUPED) {
-            group_state_fill(b->group, in, out);
+        if (grouped) {  // (pointers travel in the kernels' parameters: nothing to wait for)
+            const croft_status st = group_graph_fill(b->group, b->gexec[dir], dir, in, out);
+            if (st != CROFT_OK) return st;
         } else {
             for (size_t i = 0; i < b->pgrid.size(); ++i) {
                 b->staging[i].in = (const float2*)in[b->pgrid[i]];
@@ -315,8 +317,10 @@ static croft_status exec_batch(croft_plan plan, void* const* in, void* const* ou
             }
         }
         if (cudaGraphLaunch(b->gexec[dir], s) != cudaSuccess) { cudaGetLastError(); return CROFT_ERR_CUDA; }
-        if (cudaEventRecord(b->staging_free, s) != cudaSuccess) { cudaGetLastError(); return CROFT_ERR_CUDA; }
-        b->staging_pending = true;
+        if (!grouped) {
+            if (cudaEventRecord(b->staging_free, s) != cudaSuccess) { cudaGetLastError(); return CROFT_ERR_CUDA; }
+            b->staging_pending = true;
+        }
     }
     for (size_t i = 0; i < b->sgrid.size(); ++i) {
         const int g = b->sgrid[i];
@@ -410,8 +414,6 @@ static croft_status configure(BatchState* b, int mode) {
             croft_status st = group_state_build(b->dims, b->pgrid, &b->group);
             if (st != CROFT_OK) return st;
         }
-        if (!b->staging_free && cudaEventCreateWithFlags(&b->staging_free, cudaEventDisableTiming) != cudaSuccess)
-            return CROFT_ERR_CUDA;
     } else if (!b->d_items && !b->pgrid.empty()) {
         croft_status st = build_persistent(b);
         if (st != CROFT_OK) return st;

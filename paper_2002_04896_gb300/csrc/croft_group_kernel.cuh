@@ -7,7 +7,10 @@
 // independent and run concurrently (sibling nodes of a CUDA graph).  Each kernel
 // is the single-grid pass kernel specialised on N (compile-time radix schedule
 // and tile width) with a per-CTA lookup of its grid: CTA b works on tile
-// b - first_tile of segment cta_seg[b].
+// b - first_tile of the last segment with first_tile <= b.  The segments lie in the kernel's
+// parameters (constant bank; up to kGroupSegs of them, a pass with more grids of a length takes another launch)
+// and are searched there: a few hundred cycles less before a CTA's first load than a map and a table in memory,
+// two dependent loads - 9 % of the life of a CTA of a short pass.
 #pragma once
 #include "croft_fft_core.cuh"
 #include "croft_internal.h"
@@ -20,17 +23,27 @@ struct GroupSeg {
     float2* out;
     long long M;        // element stride of the axis (1 for a ROW pass)
     long long ncols;    // pencils of this grid along the axis
-    int first_tile;     // first CTA of this grid in the launch
     CroftColDiv cdiv;   // COL: col / M as a multiply-high (croft_coldiv.h; m = 0: divide)
 };
 
+constexpr int kGroupSegs = 32;  // a power of two
+
 struct GroupArgs {
-    const GroupSeg* segs;           // this launch's segments (device table, pointers filled per exec)
-    const unsigned short* cta_seg;  // segment of each CTA
     const float2* tw;               // twiddle table of N (two-stage: N entries; else N-1)
     int W;                          // ROW, not two-stage: pencils per CTA
     float isign;                    // +1 forward, -1 backward
+    int first_tile[kGroupSegs];     // first CTA of each grid in the launch (INT_MAX past the last)
+    GroupSeg seg[kGroupSegs];
 };
+
+// The segment of this CTA (binary search; the same in all threads).
+__device__ __forceinline__ int group_seg(const GroupArgs& A) {
+    int k = 0;
+#pragma unroll
+    for (int step = kGroupSegs / 2; step >= 1; step /= 2)
+        if (A.first_tile[k + step] <= (int)blockIdx.x) k += step;
+    return k;
+}
 
 // Batch row and column of pencil `col` of a COL segment.
 __device__ __forceinline__ long long group_col_base(const GroupSeg& S, long long col, int n) {
@@ -61,8 +74,9 @@ __global__ void __launch_bounds__(group_two<LAYOUT, N>().w* group_two<LAYOUT, N>
     C* buf = two_smem + (K.stage ? croft_two_pad(N) : 0);
     pdl_allow_dependents();
     const C* tw = two_twiddles<N, K.stage != 0>(A.tw, two_smem, K.w * K.t);
-    const GroupSeg S = A.segs[A.cta_seg[blockIdx.x]];
-    const long long tile = (long long)blockIdx.x - S.first_tile;
+    const int k = group_seg(A);
+    const GroupSeg& S = A.seg[k];
+    const long long tile = (int)blockIdx.x - A.first_tile[k];
     pdl_wait();
     if constexpr (LAYOUT == LAYOUT_ROW) {
         const int c = threadIdx.x / K.t, lane = threadIdx.x % K.t;
@@ -93,10 +107,9 @@ __global__ void __launch_bounds__(256) croft_group_kernel(const __grid_constant_
     pdl_allow_dependents();
     if (croft_make_sched(N).count > 1)
         for (int i = threadIdx.x; i < N - 1; i += blockDim.x) stw[i] = A.tw[i];
-    // (the segment table is uploaded before the first pass starts; the grid is written by
-    // the previous pass, whose launches reach this one over programmatic graph edges)
-    const GroupSeg S = A.segs[A.cta_seg[blockIdx.x]];
-    const long long tile = (long long)blockIdx.x - S.first_tile;
+    const int k = group_seg(A);
+    const GroupSeg& S = A.seg[k];
+    const long long tile = (int)blockIdx.x - A.first_tile[k];
     pdl_wait();
     if constexpr (LAYOUT == LAYOUT_ROW) {
         const int c = threadIdx.x / T;
