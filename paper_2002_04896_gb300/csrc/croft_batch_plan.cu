@@ -11,8 +11,9 @@
 //                that has it (croft_batch_group.cu), the launches of a pass
 //                concurrent.
 // ONE_LAUNCH, PER_PASS and GROUPED are recorded once into a CUDA graph per direction
-// (descriptor upload from pinned memory, counter reset, kernel launch(es));
-// an exec fills in the grids' pointers and launches the graph.  AUTO times the
+// (kernel launch(es), before them the descriptor upload from pinned memory and the
+// counter reset where the schedule has them: GROUPED carries its pointers in the
+// kernels' parameters); an exec fills in the grids' pointers and launches the graph.  AUTO times the
 // four schedules on scratch buffers at plan creation and keeps the fastest,
 // caching the choice on disk (like FFTW wisdom) keyed by the batch's sizes, the
 // GPU name and the CUDA runtime version.
@@ -220,7 +221,7 @@ static BatchArgs batch_args(const BatchState* b, int launch, int begin, int end,
     return A;
 }
 
-// Graph per direction: [descriptor upload] + [counter reset] -> kernel launch(es).
+// Graph per direction: [descriptor upload] + [counter reset] -> kernel launch(es); GROUPED: kernel launches only.
 static croft_status build_graphs(BatchState* b) {
     for (int d = 0; d < 2; ++d) {
         if (b->gexec[d]) cudaGraphExecDestroy(b->gexec[d]);
