@@ -153,7 +153,7 @@ __device__ __forceinline__ void conv_body(const C* in, C* out, const typename Cx
     col_split(col, A, b, m);
     const long long base = b * (long long)N * A.M + m;
 
-    pdl_allow_dependents();
+    if constexpr (sizeof(C) == 8) pdl_allow_dependents();  // (complex128: see pass_body)
     if (ok)
         for (int a = lane; a < N; a += T) conv_cp_async(gtile + a * W + c, g + base + (long long)a * A.M);
     asm volatile("cp.async.commit_group;" ::: "memory");

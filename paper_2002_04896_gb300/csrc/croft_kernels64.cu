@@ -13,8 +13,9 @@ namespace croft {
 
 template <int N>
 static pass64_fn col64_kernel(int w) {
-    constexpr int W = croft_col_width(N, 16);
-    return (w == W || w == 0) ? croft_pass_kernel<LAYOUT_COL, N, double2, W> : nullptr;
+    constexpr int W = croft_col_width(N, 16), H = croft_col_half64(N);  // (H = W: no narrower tile)
+    if (w == W || w == 0) return croft_pass_kernel<LAYOUT_COL, N, double2, W>;
+    return w == H ? croft_pass_kernel<LAYOUT_COL, N, double2, H> : nullptr;
 }
 
 pass64_fn pass64_kernel_for(int layout, int n, int w) {
