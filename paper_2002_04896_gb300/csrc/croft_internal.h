@@ -206,6 +206,9 @@ cudaError_t launch_scale(const void* in, void* out, const void* g, long long n, 
 
 // croft_passes.cu
 extern int g_max_smem;  // the device's opt-in shared memory per block (set by plan creation)
+// Lets launches of kernel f take `bytes` of dynamic shared memory.  The limit belongs to the function, not to a plan:
+// every plan whose pass runs f launches under it, so it is raised where it is too low and never lowered.
+cudaError_t allow_smem(const void* f, int bytes);
 // Launch shape of one axis pass (tile width, block, grid, shared memory); false when no shape fits.
 bool shape_pass(PassLaunch& L, int layout, int n, long long M, long long ncols, int tc = 0, bool f64 = false,
                 int want_w = 0, int sv = 0, int th = 0);

@@ -77,6 +77,16 @@ bool shape_pass(PassLaunch& L, int layout, int n, long long M, long long ncols, 
     return true;
 }
 
+cudaError_t allow_smem(const void* f, int bytes) {
+    if (bytes <= 48 * 1024) return cudaSuccess;  // (what every kernel may take)
+    static std::mutex m;  // plans are created in several threads: look and raise as one step
+    std::lock_guard<std::mutex> lock(m);
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, f);
+    if (e != cudaSuccess || a.maxDynamicSharedSizeBytes >= bytes) return e;
+    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no link to libcuda).
 static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
     static std::once_flag once;

@@ -17,7 +17,7 @@ plane_pass_fn plane_pass_kernel_for(int ny) {
 cudaError_t plane_pass_prepare(int ny, int smem) {
     plane_pass_fn f = plane_pass_kernel_for(ny);
     if (!f) return cudaErrorInvalidValue;
-    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    return allow_smem((const void*)f, smem);
 }
 
 cudaError_t launch_plane_pass(const PlanePass& P, const float2* in, float2* out, float isign, cudaStream_t s, bool pdl) {
