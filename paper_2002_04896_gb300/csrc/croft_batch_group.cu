@@ -128,7 +128,7 @@ croft_status group_state_build(const std::vector<int>& dims, const std::vector<i
             L.nseg = L.ctas = 0;
             memset(&L.args, 0, sizeof(L.args));
             for (int& t : L.args.first_tile) t = INT_MAX;
-            if (L.smem > 48 * 1024 && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, L.smem) != cudaSuccess) {
+            if (allow_smem((const void*)f, L.smem) != cudaSuccess) {
                 cudaGetLastError();
                 group_state_destroy(s);
                 return CROFT_ERR_CUDA;

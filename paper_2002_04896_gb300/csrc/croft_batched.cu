@@ -122,8 +122,7 @@ int batch_smem_bytes() {
 }
 
 cudaError_t batched_prepare(int smem) {
-    if (smem <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(croft_batched_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    return allow_smem((const void*)croft_batched_kernel, smem);
 }
 
 int batched_blocks_per_sm(int smem) {

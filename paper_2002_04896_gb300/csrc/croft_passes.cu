@@ -157,7 +157,7 @@ bool shape_pair(PassLaunch& L, int n, long long M, long long ncols) {
     const long long grid = 2 * ((ncols + kPairTileWidth - 1) / kPairTileWidth);
     if (grid > 0x7fffffffLL || L.smem > g_max_smem) return false;
     L.grid = (int)grid;
-    if (L.smem > 48 * 1024 && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, L.smem) != cudaSuccess) {
+    if (allow_smem((const void*)f, L.smem) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
@@ -198,7 +198,7 @@ bool shape_ring(PassLaunch& L, int n, long long M, long long ncols) {
     L.block = 1024;
     L.smem = (R.tw_pad + 3 * n * kRingTileWidth) * (int)sizeof(float2) + 128;  // + alignment of the tiles
     if (L.smem > g_max_smem) return false;
-    if (L.smem > 48 * 1024 && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, L.smem) != cudaSuccess) {
+    if (allow_smem((const void*)f, L.smem) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
@@ -243,7 +243,7 @@ void shape_two(TwoLaunch& two, int layout, int n, long long M, long long ncols) 
     const int smem = croft_two_smem(K, n, row);
     const long long grid = (ncols + K.w - 1) / K.w * K.ctas;
     if (smem > g_max_smem || grid > 0x7fffffffLL) return;
-    if (smem > 48 * 1024 && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
+    if (allow_smem((const void*)f, smem) != cudaSuccess) {
         cudaGetLastError();
         return;
     }
@@ -303,7 +303,7 @@ bool pass_supports_pdl(const PassLaunch& L) { return !L.tc || croft_tc_two(L.arg
 
 cudaError_t prepare_pass(const PassLaunch& L) {
     if (L.kind == PASS_PLANE) {
-        cudaError_t e = cudaFuncSetAttribute(L.pk.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, L.smem);
+        cudaError_t e = allow_smem((const void*)L.pk.fn, L.smem);
         if (e != cudaSuccess) return e;
         if (L.pk.cluster > 8) {
             e = cudaFuncSetAttribute(L.pk.fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -321,19 +321,16 @@ cudaError_t prepare_pass(const PassLaunch& L) {
     if (L.ring) {
         ring_fn f = ring_kernel_for(L.args.n);
         if (!f || !tensor_map_encoder()) return cudaErrorInvalidValue;
-        if (L.smem <= 48 * 1024) return cudaSuccess;
-        return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, L.smem);
+        return allow_smem((const void*)f, L.smem);
     }
     if (L.f64) {
         pass64_fn f = pass64_kernel_for(L.layout, L.args.n, L.args.W);
         if (!f) return cudaErrorInvalidValue;
-        if (L.smem <= 48 * 1024) return cudaSuccess;
-        return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, L.smem);
+        return allow_smem((const void*)f, L.smem);
     }
     pass_fn f = L.tc ? tc_pass_kernel_for(L.layout, L.args.n, L.tc - 1) : pass_kernel_for(L.layout, L.args.n, L.args.W, L.sv, L.th);
     if (!f) return cudaErrorInvalidValue;
-    if (L.smem <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, L.smem);
+    return allow_smem((const void*)f, L.smem);
 }
 
 cudaError_t launch_pass(const PassLaunch& L, const void* vin, void* vout, cudaStream_t s, bool pdl) {

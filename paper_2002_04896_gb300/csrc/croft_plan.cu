@@ -522,7 +522,7 @@ static void plan_conv(croft_plan p) {
         cudaGetLastError();
         return;
     }
-    if (L.smem > 48 * 1024 && cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, L.smem) != cudaSuccess) {
+    if (allow_smem(fn, L.smem) != cudaSuccess) {
         cudaGetLastError();
         return;
     }

@@ -35,3 +35,17 @@ def test_plane_pass_plans(croft_lib, older, newer):
             assert oracle.rel_l2(y.cpu().numpy(), oracle.forward(x)) <= tol, shape
             assert oracle.rel_l2(z.cpu().numpy(), oracle.backward(x)) <= tol, shape
             assert oracle.rel_l2(c.cpu().numpy(), x.size * x.astype(np.complex128)) <= 2 * tol, shape
+
+
+# complex128 rows of 1024 points: full tiles of the older plan, half tiles of the newer one
+def test_complex128_row_plans(croft_lib):
+    older, newer = (64, 64, 1024), (96, 64, 1024)
+    f64 = croft_lib.CROFT_C2C_F64
+    with croft_lib.Plan(*older, dtype=f64) as a, croft_lib.Plan(*newer, dtype=f64) as b:
+        for plan, shape in ((a, older), (b, newer), (a, older)):
+            x = torch.from_numpy(_input(shape, 7, np.complex128)).cuda()
+            y = torch.empty_like(x)
+            croft_lib.croft_exec_axes(plan.handle, x, y, 4, -1)  # the z axis
+            torch.cuda.synchronize()
+            e = oracle.rel_l2(y[::16].cpu().numpy(), oracle.dft_along_axis(x[::16].cpu().numpy(), 2, -1))
+            assert e <= 1e-14 * math.log2(1024), (shape, e)
