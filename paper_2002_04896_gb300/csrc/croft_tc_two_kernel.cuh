@@ -11,8 +11,10 @@
 // What bounds it: the latency of that chain at three or four 256-thread CTAs per SM (five barriers and an MMA round trip
 // in it); the tensor pipe idles.  Against three stages (16, then the near-equal split of the rest: one exchange and
 // two barriers more, at 32 threads per pencil) a 512^3 bf16x3 forward transform went from 1630 to 1364 us, 256^3 from 184 to 149.
-// The next pass may become resident while this one drains (programmatic dependent launch): all of this
-// launch's CTAs run by then, so a waiting CTA's TMEM allocation delays none of them.
+// The next pass may become resident while this one drains (programmatic dependent launch).  Its CTAs hold TMEM
+// while they wait for this pass to end, so no CTA of this pass may still want TMEM then: the warp that allocates
+// it lets the dependents start only after it has it.  (Allowed earlier, a dependent on the same SM could take the columns that a
+// CTA of this pass waits for, beside another program's kernel that holds the rest, and neither would end.)
 #pragma once
 #include "croft_tc_kernel.cuh"
 #include "croft_two_stage_kernel.cuh"
@@ -53,7 +55,9 @@ __global__ void __launch_bounds__(256, tc_two_minb(N)) croft_tc_two_kernel(const
     unsigned char* bmat = (unsigned char*)smem;
     unsigned char* ops = bmat + 4096;  // group (q, g): hi 8 KB at (2 * (2 * q + g)) * 8192, lo behind it
     const int tid = threadIdx.x, g = tid >> 7, row = tid & 127;
-    pdl_allow_dependents();
+    // CTAs of such passes that an SM's shared memory (228 KB, 1 KB of it reserved per CTA) holds never want more than its
+    // 512 columns together, whatever their lengths, so the allocation waits only for other kernels
+    static_assert((tc_two_smem(N, LAYOUT == LAYOUT_ROW) + 1024) * 512 >= NCOLS * 228 * 1024, "TMEM columns per SM");
     ((uint4*)bmat)[tid] = ((const uint4*)A.tc_b)[tid];
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&mbar)));
@@ -62,6 +66,7 @@ __global__ void __launch_bounds__(256, tc_two_minb(N)) croft_tc_two_kernel(const
     if (tid < 32) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tmem_slot)), "r"(NCOLS));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+        pdl_allow_dependents();  // (by this warp alone: not before the allocation)
     }
 
     int c, lane;
