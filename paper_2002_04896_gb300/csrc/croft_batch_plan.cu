@@ -353,7 +353,8 @@ static std::string tune_key(const BatchState* b) {
     cudaDeviceProp prop;
     cudaGetDeviceProperties(&prop, dev);
     char buf[512];
-    snprintf(buf, sizeof(buf), "batch-v2:%d:%016llx:%s:%d", b->count, h, prop.name, rt);
+    // (":two-stage": the kernels that the schedules were timed with)
+    snprintf(buf, sizeof(buf), "batch-v2:%d:%016llx:%s:%d:two-stage", b->count, h, prop.name, rt);
     for (char* c = buf; *c; ++c)
         if (*c == ' ' || *c == '"') *c = '_';
     return buf;

@@ -130,6 +130,23 @@ def test_autotune_chooses_and_caches(croft_lib, pme_batch, tmp_path, monkeypatch
     assert len(cache.read_text().strip().splitlines()) == 1
 
 
+def test_autotune_measures_again_where_the_choice_is_of_older_kernels(croft_lib, tmp_path, monkeypatch):
+    """A choice saved under the key of the three-stage kernels (no suffix after the runtime version) is not taken."""
+    dims = [(48, 40, 36), (36, 48, 40)]
+    cache = tmp_path / "tune.txt"
+    monkeypatch.setenv("CROFT_TUNE_CACHE", str(cache))
+    monkeypatch.delenv("CROFT_TUNE", raising=False)
+    with croft_lib.BatchPlan(dims):
+        pass
+    key = cache.read_text().split()[0]
+    old = ":".join(key.split(":")[:5])
+    cache.write_text(f"{old} 1 one_launch_us=1.0 per_pass_us=9.0 per_grid_us=9.0 grouped_us=9.0\n")
+    with croft_lib.BatchPlan(dims):
+        pass
+    lines = cache.read_text().strip().splitlines()
+    assert len(lines) == 2 and lines[1].split()[0] == key != old
+
+
 def test_bounded_wait_times_out_with_status_and_context_survives(croft_lib, mixed_inputs):
     """A dependency count nothing reaches: the waits give up after the limit, status TIMEOUT, no hang."""
     ins = [torch.from_numpy(x).cuda() for x in mixed_inputs]
