@@ -227,16 +227,20 @@ static int rules_sv(croft_plan p, int axis) {
     return croft_col_sv_default(n, 8, M * 8);
 }
 
-// Gives pass L over the axis its two-stage kernel where the length has one (croft_two_stage.h): the
-// complex64 CUDA-core passes that the rules plan.  A tuned plan's choice and the measurement switches
-// CROFT_RING, CROFT_PAIR and CROFT_COL_TH name a kernel and keep it; CROFT_TWO_STAGE=0 switches the
+// Whether the rules give an axis's passes two-stage kernels (croft_two_stage.h) where the length has one: the
+// complex64 CUDA-core passes.  A tuned plan's choice names a kernel and keeps it; so do the measurement
+// switches CROFT_RING, CROFT_PAIR and CROFT_COL_TH for the passes that they give one.  CROFT_TWO_STAGE=0 switches the
 // two-stage kernels off.
+static bool two_selected(croft_plan p, int axis) {
+    const char* te = getenv("CROFT_TWO_STAGE");
+    return p->dtype != CROFT_C2C_F64 && !p->axis_tc[axis] && p->axis_kind[axis] < 0 && !(te && te[0] == '0') &&
+           !getenv("CROFT_RING") && !getenv("CROFT_PAIR") && !getenv("CROFT_COL_TH");
+}
+
+// Gives pass L over the axis its two-stage kernel where there is one for it.
 static void attach_two(croft_plan p, int axis, PassLaunch& L) {
     memset(&L.two, 0, sizeof(L.two));
-    const char* te = getenv("CROFT_TWO_STAGE");
-    if (L.f64 || L.tc || p->axis_kind[axis] >= 0 || (te && te[0] == '0') || getenv("CROFT_RING") || getenv("CROFT_PAIR") ||
-        getenv("CROFT_COL_TH"))
-        return;
+    if (!two_selected(p, axis)) return;
     shape_two(L.two, L.layout, L.args.n, L.args.M, L.args.ncols);
     if (!L.two.fn) return;
     const int n = L.args.n;
@@ -260,10 +264,12 @@ static croft_status add_axis_pass(croft_plan p, int axis, int x0 = 0, int nxs = 
     // pass, CROFT_RING=0 for none (both for measurement).
     const int kind = p->axis_kind[axis];
     const bool ring_pass = layout == LAYOUT_COL && ring_selected(p, axis);
-    // The cluster-pair kernel (croft_pair_kernel.cuh): tuned plans (kind 2) or CROFT_PAIR=1.
+    // The cluster-pair kernel (croft_pair_kernel.cuh): tuned plans (kind 2), CROFT_PAIR=1, or the rule
+    // (croft_pair_default) where the two-stage kernels are off.
     const char* pe = getenv("CROFT_PAIR");
-    const bool pair_pass = layout == LAYOUT_COL && !f64 && !p->axis_tc[axis] && !ring_pass &&
-                           (kind >= 0 ? kind == 2 : (pe ? pe[0] == '1' : croft_pair_default(n, 8, M * 8)));
+    const bool pair_pass =
+        layout == LAYOUT_COL && !f64 && !p->axis_tc[axis] && !ring_pass &&
+        (kind >= 0 ? kind == 2 : (pe ? pe[0] == '1' : !two_selected(p, axis) && croft_pair_default(n, 8, M * 8)));
     if (pair_pass) {
         PassLaunch L;
         if (shape_pair(L, n, M, N / n)) {
@@ -289,8 +295,7 @@ static croft_status add_axis_pass(croft_plan p, int axis, int x0 = 0, int nxs = 
             L.offset = offset;
             L.src_in = sin;
             L.group = grp;
-            attach_two(p, axis, L);
-            if (L.two.fn || prepare_pass(L) == cudaSuccess) {
+            if (prepare_pass(L) == cudaSuccess) {
                 p->passes.push_back(L);
                 p->pass_axis.push_back(axis);
                 if (grp >= p->ngroups) p->ngroups = grp + 1;

@@ -38,6 +38,12 @@ def test_single_grid_plan_oom_at_every_allocation(croft_lib):
     assert _sweep(croft_lib, lambda: croft_lib.croft_plan_create_status(64, 48, 40)) == 3  # one table per axis
 
 
+def test_no_table_for_a_kernel_that_does_not_run(croft_lib):
+    # lengths of the cluster-pair rule, whose passes run two-stage kernels: one table per axis
+    for shape in ((512, 256, 256), (500, 256, 256), (486, 45, 50), (3, 486, 50)):
+        assert _sweep(croft_lib, lambda: croft_lib.croft_plan_create_status(*shape)) == 3, shape
+
+
 def test_tensor_core_plan_oom_at_every_allocation(croft_lib):
     n = _sweep(croft_lib, lambda: croft_lib.croft_plan_create_status(4, 256, 512, croft_lib.CROFT_C2C_F32_TC_BF16X3))
     assert n == 5  # DFT-16 operand, status word, three twiddle tables

@@ -2,9 +2,9 @@
 
 Two CTAs of a 2-CTA cluster share a 16-column tile of an even 270..512-point axis: each
 transforms the even or the odd rows at half length, and a radix-2 step across the pair
-(one operand read through distributed shared memory) combines them.  By default it runs the
-512-point passes across strides of 256 KB or more (the 512^3 x pass); CROFT_PAIR=1 selects it
-for every column pass it can serve; tuned plans may pick it.  Every length as x and y,
+(one operand read through distributed shared memory) combines them.  CROFT_PAIR=1 selects it
+for every column pass it can serve; tuned plans may pick it; where the two-stage kernels are off
+(CROFT_TWO_STAGE=0) a rule takes it, for 512-point passes across strides of 256 KB or more among others.  Every length as x and y,
 ragged tiles, forward and backward, in place, determinism.
 """
 
@@ -37,6 +37,12 @@ def pair_on():
         os.environ["CROFT_PAIR"] = old
 
 
+@pytest.fixture()
+def general_kernels(monkeypatch):
+    """The kernels that run where the two-stage ones are off."""
+    monkeypatch.setenv("CROFT_TWO_STAGE", "0")
+
+
 def _noise(shape, seed):
     rng = np.random.default_rng(seed)
     return (rng.uniform(-1, 1, shape) + 1j * rng.uniform(-1, 1, shape)).astype(np.complex64)
@@ -50,6 +56,8 @@ def _check(croft, x, n_pair_passes):
         yb = p.backward(d)
         torch.cuda.synchronize()
     assert desc.count("+pair") == n_pair_passes, desc
+    # (what stands behind "->" is the kernel that runs)
+    assert not any("+pair" in part and "->" in part for part in desc.split(" | ")), desc
     t = tol(x.shape)
     ef = oracle.rel_l2(yf.cpu().numpy(), oracle.forward(x))
     eb = oracle.rel_l2(yb.cpu().numpy(), oracle.backward(x))
@@ -83,8 +91,8 @@ def test_pair_not_for_odd_lengths(croft_lib, pair_on):
     _check(croft_lib, _noise((375, 2, 1350), 3), 0)
 
 
-def test_pair_default_for_512_point_long_strides(croft_lib):
-    """Without CROFT_PAIR: the x pass of a 512 x 256 x 256 grid (512 KB strides) is a pair pass,
+def test_pair_default_for_512_point_long_strides(croft_lib, general_kernels):
+    """By the rule, two-stage kernels off: the x pass of a 512 x 256 x 256 grid (512 KB strides) is a pair pass,
     its y pass (2 KB) and a 512 x 128 x 128 grid's x pass (128 KB) are not."""
     x = _noise((512, 256, 256), 11)
     ref = oracle.forward(x)
@@ -93,14 +101,14 @@ def test_pair_default_for_512_point_long_strides(croft_lib):
         desc = p.describe()
         y = p.forward(d)
         torch.cuda.synchronize()
-    assert desc.count("+pair") == 1 and "x:col+pair" in desc, desc
+    assert desc.count("+pair") == 1 and "x:col+pair" in desc and "two-stage" not in desc, desc
     assert oracle.rel_l2(y.cpu().numpy(), ref) <= tol(x.shape)
     with croft_lib.Plan(512, 128, 128) as p:
         assert "+pair" not in p.describe()
 
 
-def test_pair_default_for_486_and_500(croft_lib):
-    """Without CROFT_PAIR: 486-point passes pair at every stride (y across 40 bytes, x across
+def test_pair_default_for_486_and_500(croft_lib, general_kernels):
+    """By the rule, two-stage kernels off: 486-point passes pair at every stride (y across 40 bytes, x across
     18 KB), 500-point ones only across 256 KB or more."""
     with croft_lib.Plan(486, 45, 50) as p:
         d = p.describe()

@@ -113,10 +113,11 @@ def test_16_thread_pencils_by_default_for_432_and_480_across_long_strides(croft_
             assert " T=32 " in _pass_desc(p.describe(), "x"), p.describe()
 
 
-def test_column_width_follows_the_stride(croft_lib, dev):
-    """512^3: the y pass (4 KB stride) runs 8-column tiles, the x pass (2 MB stride) 16-column
+def test_column_width_follows_the_stride(croft_lib, dev, monkeypatch):
+    """General kernels, 512^3: the y pass (4 KB stride) runs 8-column tiles, the x pass (2 MB stride) 16-column
     tiles split over a cluster pair of 256-thread CTAs; below 256 KB strides the plain
     16-column, 512-thread tile."""
+    monkeypatch.setenv("CROFT_TWO_STAGE", "0")
     with croft_lib.Plan(512, 512, 512) as p:
         d = p.describe()
     assert " W=8 block=256 " in _pass_desc(d, "y"), d
