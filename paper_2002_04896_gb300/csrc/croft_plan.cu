@@ -228,13 +228,11 @@ static int rules_sv(croft_plan p, int axis) {
 }
 
 // Whether the rules give an axis's passes two-stage kernels (croft_two_stage.h) where the length has one: the
-// complex64 CUDA-core passes.  A tuned plan's choice names a kernel and keeps it; so do the measurement
-// switches CROFT_RING, CROFT_PAIR and CROFT_COL_TH for the passes that they give one.  CROFT_TWO_STAGE=0 switches the
+// complex64 CUDA-core passes.  A tuned plan's choice names a kernel and keeps it; CROFT_TWO_STAGE=0 switches the
 // two-stage kernels off.
 static bool two_selected(croft_plan p, int axis) {
     const char* te = getenv("CROFT_TWO_STAGE");
-    return p->dtype != CROFT_C2C_F64 && !p->axis_tc[axis] && p->axis_kind[axis] < 0 && !(te && te[0] == '0') &&
-           !getenv("CROFT_RING") && !getenv("CROFT_PAIR") && !getenv("CROFT_COL_TH");
+    return p->dtype != CROFT_C2C_F64 && !p->axis_tc[axis] && p->axis_kind[axis] < 0 && !(te && te[0] == '0');
 }
 
 // Gives pass L over the axis its two-stage kernel where there is one for it.
@@ -327,8 +325,9 @@ static croft_status add_axis_pass(croft_plan p, int axis, int x0 = 0, int nxs = 
     // CROFT_COL_TH=16 (measurement): 16-column tiles with 16 threads per pencil for every column
     // pass of 32-thread pencils that a plan's rules would give the plain kernel
     const char* te = getenv("CROFT_COL_TH");
-    if (kind < 0 && te && atoi(te) == 16 && layout == LAYOUT_COL && !f64 && !p->axis_tc[axis] &&
-        croft_threads_per_pencil(n) == 32) {
+    const bool th_named = kind < 0 && te && atoi(te) == 16 && layout == LAYOUT_COL && !f64 && !p->axis_tc[axis] &&
+                          croft_threads_per_pencil(n) == 32;
+    if (th_named) {
         th = 16;
         want_w = croft_col_width(n, 8);
     }
@@ -356,7 +355,7 @@ static croft_status add_axis_pass(croft_plan p, int axis, int x0 = 0, int nxs = 
     L.offset = offset;
     L.src_in = sin;
     L.group = grp;
-    attach_two(p, axis, L);
+    if (!th_named) attach_two(p, axis, L);
     if (!L.two.fn && prepare_pass(L) != cudaSuccess) return CROFT_ERR_CUDA;
     p->passes.push_back(L);
     p->pass_axis.push_back(axis);

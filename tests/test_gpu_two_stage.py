@@ -72,3 +72,19 @@ def test_convolution_with_ragged_tiles(croft_lib, n):
         assert torch.equal(torch.view_as_real(y), torch.view_as_real(d))
         e = oracle.rel_l2(y.cpu().numpy(), oracle.convolve(x, g))
         assert e <= 4e-6 * math.log2(x.size), (shape, e)
+
+
+@pytest.mark.parametrize("switch,kernel,two", [(None, None, 3), ("CROFT_RING=0", None, 3), ("CROFT_PAIR=0", None, 3),
+                                               ("CROFT_RING=1", "+ring", 2), ("CROFT_PAIR=1", "+pair", 2),
+                                               ("CROFT_COL_TH=16", " T=16 ", 2), ("CROFT_TWO_STAGE=0", None, 0)])
+def test_switches_name_their_own_kernels_only(croft_lib, monkeypatch, switch, kernel, two):
+    """A measurement switch that names a kernel takes it for the passes it can serve (here x) and leaves the others
+    alone; one that rules a kernel out leaves the two-stage kernels alone."""
+    if switch:
+        monkeypatch.setenv(*switch.split("="))
+    with croft_lib.Plan(480, 36, 512) as p:
+        d = p.describe()
+    x = [s for s in d.split(" | ") if s.startswith("x:")][0]
+    assert d.count("-> two-stage") == two, d
+    assert ("-> two-stage" in x) == (kernel is None and two > 0), d
+    assert kernel is None or kernel in x, d
