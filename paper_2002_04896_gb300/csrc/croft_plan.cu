@@ -243,7 +243,9 @@ static void attach_two(croft_plan p, int axis, PassLaunch& L) {
     if (!L.two.fn) return;
     const int n = L.args.n;
     L.two.tw = p->tw_dev[axis] + n;  // (the axis's second table)
+    if (p->tw_two[axis] == L.two.r1) return;  // (the slab schedule runs an axis slab by slab: one table for all)
     host_build_two_twiddles(n, L.two.r1, p->tw_host[axis].data() + 2 * (size_t)n);
+    p->tw_two[axis] = L.two.r1;
 }
 
 static croft_status add_axis_pass(croft_plan p, int axis, int x0 = 0, int nxs = -1, int group = -1, int src_in = -1) {
@@ -578,6 +580,7 @@ static croft_status create_impl(croft_plan* out, int nx, int ny, int nz, croft_d
     for (int a = 0; a < 3; ++a) {
         p->tw_dev[a] = NULL;
         p->tw_pair[a] = NULL;
+        p->tw_two[a] = 0;
     }
     p->timing = false;
     p->ev_count = 0;

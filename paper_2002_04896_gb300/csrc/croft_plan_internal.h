@@ -26,6 +26,7 @@ struct croft_plan_s {
                                       // (complex64) n entries each for its two-stage kernel, the plane
                                       // pass and the fused convolution
     CroftSched tw_sched[3];           // complex64: the schedule of the axis's own table (count 0: none or built already)
+    int tw_two[3];                    // first radix of the axis's second table (0: not built)
     std::vector<float> tw_host[3];    // complex64 tables until their upload at the end of creation
     croft::PlanePass zy;              // z and y in one pass over the planes (fn NULL: axis by axis)
     float2* tw_pair[3];               // pair column passes: [half-length table | combine twiddles], else NULL
