@@ -299,6 +299,7 @@ croft_status croft_exec_backward(croft_plan plan, const void* in, void* out, voi
  *
  *   plan      : a single-grid plan with one pass per axis (CROFT_SCHEDULE_THREE_PASS and
  *               AUTO); the fused-plane and slab schedules give CROFT_ERR_INVALID_ARG.
+ *               All three axes in one call give the bits of croft_exec_forward / _backward.
  *   in, out   : device pointers as for croft_exec_forward (in == out allowed).
  *   axes      : bit a set to transform axis a (0 = x, 1 = y, 2 = z); 0 copies in to out.
  *   direction : -1 forward (Eq. 1), +1 backward (Eq. 2, unnormalised).
@@ -398,8 +399,8 @@ int croft_plan_describe(croft_plan plan, char* buf, int cap);
  * Per-pass timing (tracing hook).  When enabled, each exec records a CUDA
  * event on the exec stream before the first pass and after every logical pass
  * (the slab schedule's z+y launches count as one pass).  While it is enabled every axis
- * runs a pass of its own, also where an AUTO plan otherwise runs z and y as one (the same
- * transform, rounded differently).
+ * runs a pass of its own, also where an AUTO plan otherwise runs z and y as one (with the
+ * same bits).
  * croft_plan_pass_times waits for the last exec's events and writes the
  * duration in milliseconds of each pass into ms[0 .. min(cap, passes)-1];
  * it returns the number of passes timed, 0 when timing is off or no exec ran,

@@ -408,12 +408,12 @@ static croft_status plan_zy(croft_plan p) {
     }
     for (int axis = 1; axis <= 2; ++axis) {
         const int n = p->dims[axis];
-        host_build_two_twiddles(n, croft_plane_r1(n), p->tw_host[axis].data() + 4 * (size_t)n);
+        host_build_two_twiddles(n, croft_plane_axis(n, axis == 2).r1, p->tw_host[axis].data() + 4 * (size_t)n);
     }
     z.args.tw_z = p->tw_dev[2] + 2 * nz;
     z.args.tw_y = p->tw_dev[1] + 2 * ny;
     z.args.nz = nz;
-    z.args.r1z = croft_plane_r1(nz);
+    z.args.r1z = croft_plane_r1z(nz);
     z.args.pitch = croft_plane_pitch(nz);
     z.args.ld = croft_plane_ld(nz);
     z.args.div_nz = (unsigned)((0x100000000ull + (unsigned)nz - 1) / (unsigned)nz);
@@ -1009,8 +1009,8 @@ int croft_plan_describe(croft_plan plan, char* buf, int cap) {
     }
     if (plan->zy.fn) {
         snprintf(tmp, sizeof(tmp), " | z+y in one pass over the planes: %dx%d, %dx%d block=%d grid=%d smem=%d",
-                 croft_plane_r1(plan->dims[2]), plan->dims[2] / croft_plane_r1(plan->dims[2]), croft_plane_r1(plan->dims[1]),
-                 plan->dims[1] / croft_plane_r1(plan->dims[1]), plan->zy.block, plan->zy.grid, plan->zy.smem);
+                 croft_plane_r1z(plan->dims[2]), plan->dims[2] / croft_plane_r1z(plan->dims[2]), croft_plane_r1y(plan->dims[1]),
+                 plan->dims[1] / croft_plane_r1y(plan->dims[1]), plan->zy.block, plan->zy.grid, plan->zy.smem);
         s += tmp;
     }
     if (plan->conv_fused) {

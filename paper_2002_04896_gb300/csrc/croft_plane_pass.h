@@ -3,38 +3,31 @@
 #pragma once
 
 #include "croft_sched.h"
+#include "croft_two_stage.h"
 
-// First radix of a plane axis of n points, n = R1 * R2, both at most 16 (125: 25): the z and y
-// transforms of a plane take two stages each.  0: no plane kernel for the length.
-CROFT_HD constexpr int croft_plane_r1(int n) {
-    switch (n) {
-        case 32: return 8;
-        case 36: return 6;
-        case 40: return 8;
-        case 45: return 9;
-        case 48: return 8;
-        case 50: return 10;
-        case 54: return 9;
-        case 60: return 10;
-        case 64: return 8;
-        case 72: return 9;
-        case 75: return 15;
-        case 80: return 10;
-        case 81: return 9;
-        case 90: return 10;
-        case 96: return 12;
-        case 100: return 10;
-        case 108: return 12;
-        case 120: return 12;
-        case 125: return 25;
-        case 128: return 16;
-        default: return 0;
-    }
+// Whether an axis of n points may be one of a plane (both radices at most 16; 125: 25).
+CROFT_HD constexpr bool croft_plane_length(int n) {
+    return n == 32 || n == 36 || n == 40 || n == 45 || n == 48 || n == 50 || n == 54 || n == 60 || n == 64 || n == 72 ||
+           n == 75 || n == 80 || n == 81 || n == 90 || n == 96 || n == 100 || n == 108 || n == 120 || n == 125 || n == 128;
 }
+// How a plane's z and y axes split, n = R1 * R2, and whether their sums are paired: as the axis passes do (32 points: their
+// stages 16 and 2), so that a transform has the same bits whether z and y run as one pass or as two (per-axis timing,
+// croft_exec_axes, batches).
+struct CroftPlaneAxis {
+    int r1, packed;
+};
+CROFT_HD constexpr CroftPlaneAxis croft_plane_axis(int n, bool z) {
+    if (!croft_plane_length(n)) return CroftPlaneAxis{0, 0};
+    if (n == 32) return CroftPlaneAxis{16, 0};
+    const CroftTwo k = z ? croft_two_row(n) : croft_two_col(n, false);
+    return CroftPlaneAxis{k.r1, k.packed};
+}
+CROFT_HD constexpr int croft_plane_r1z(int nz) { return croft_plane_axis(nz, true).r1; }
+CROFT_HD constexpr int croft_plane_r1y(int ny) { return croft_plane_axis(ny, false).r1; }
 // Elements from one run of a z transform's second stage to the next in shared memory (odd: no bank conflicts
 // between neighbouring frequencies), and from one row of the plane to the next (odd likewise).
-CROFT_HD constexpr int croft_plane_pitch(int nz) { return (nz / croft_plane_r1(nz)) | 1; }
-CROFT_HD constexpr int croft_plane_ld(int nz) { return (croft_plane_r1(nz) * croft_plane_pitch(nz)) | 1; }
+CROFT_HD constexpr int croft_plane_pitch(int nz) { return (nz / croft_plane_r1z(nz)) | 1; }
+CROFT_HD constexpr int croft_plane_ld(int nz) { return (croft_plane_r1z(nz) * croft_plane_pitch(nz)) | 1; }
 // Shared memory: [plane: ny rows of ld][slot of every z frequency: nz 16-bit numbers].
 CROFT_HD constexpr int croft_plane_smem(int ny, int nz) { return ny * croft_plane_ld(nz) * 8 + (nz * 2 + 15) / 16 * 16; }
 
@@ -48,7 +41,7 @@ CROFT_HD constexpr int croft_plane_smem(int ny, int nz) { return ny * croft_plan
 // stays in the L2 (z and y of 960 planes, two passes / plane pass: 72^2 30.4 / 27.4 us, 80^2 35.3 / 35.8, 96^2
 // 48.4 / 54.0, 108^2 60 / 67).
 CROFT_HD constexpr bool croft_plane_pass_rule(int nx, int ny, int nz) {
-    return croft_plane_r1(ny) != 0 && croft_plane_r1(nz) != 0 &&
+    return croft_plane_length(ny) && croft_plane_length(nz) &&
            (ny * nz <= 4096 || (nx >= 288 && (ny * nz <= 6400 || (ny * nz <= 10000 && nx <= 456))));
 }
 // Threads of a plane's CTA: enough for one round of butterflies a stage where an SM holds one plane, fewer (and

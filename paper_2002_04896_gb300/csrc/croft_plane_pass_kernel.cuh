@@ -27,37 +27,40 @@
 #include "croft_fft_core.cuh"
 #include "croft_internal.h"
 #include "croft_plane_pass.h"
+#include "croft_two_stage_kernel.cuh"
 
 namespace croft {
 
 // z1 and z2 of a plane of ny rows.
 template <int NZ>
 __device__ __noinline__ void plane_z(const float2* in, const float2* tw, int ny, unsigned div_ny, float isign) {
-    extern __shared__ __align__(16) float2 plane_tile[];
-    constexpr int R1 = croft_plane_r1(NZ), R2 = NZ / R1, PITCH = croft_plane_pitch(NZ), LD = croft_plane_ld(NZ);
+    extern __shared__ __align__(16) float2 plane_raw[];
+    using C = typename TwoComplex<croft_plane_axis(NZ, true).packed != 0>::type;
+    C* plane_tile = reinterpret_cast<C*>(plane_raw);
+    constexpr int R1 = croft_plane_r1z(NZ), R2 = NZ / R1, PITCH = croft_plane_pitch(NZ), LD = croft_plane_ld(NZ);
     for (int i = threadIdx.x; i < ny * R2; i += blockDim.x) {
         const int y = i / R2, b = i - y * R2;
-        const float2* src = in + y * NZ + b;
-        float2 v[R1];
+        const C* src = reinterpret_cast<const C*>(in) + y * NZ + b;
+        C v[R1];
 #pragma unroll
         for (int j = 0; j < R1; ++j) {
             v[j] = src[j * R2];
-            v[j].y *= isign;
+            conj_if(v[j], isign);
         }
         dft<R1>(v);
-        float2* d = plane_tile + y * LD + b;
+        C* d = plane_tile + y * LD + b;
 #pragma unroll
         for (int k = 0; k < R1; ++k) d[k * PITCH] = v[k];
     }
     __syncthreads();
     for (int i = threadIdx.x; i < ny * R1; i += blockDim.x) {
         const int k = (int)__umulhi((unsigned)i, div_ny), y = i - k * ny;
-        float2* d = plane_tile + y * LD + k * PITCH;
-        float2 v[R2];
+        C* d = plane_tile + y * LD + k * PITCH;
+        C v[R2];
 #pragma unroll
         for (int j = 0; j < R2; ++j) v[j] = d[j];
 #pragma unroll
-        for (int j = 1; j < R2; ++j) v[j] = cmul(v[j], tw[j * R1 + k]);
+        for (int j = 1; j < R2; ++j) v[j] = cmul(v[j], reinterpret_cast<const C*>(tw)[j * R1 + k]);
         dft<R2>(v);
 #pragma unroll
         for (int j = 0; j < R2; ++j) d[j] = v[j];
@@ -70,9 +73,11 @@ __device__ __noinline__ void plane_z(const float2* in, const float2* tw, int ny,
 
 template <int NY>
 __global__ void __launch_bounds__(1024) croft_plane_pass_kernel(const __grid_constant__ PlanePassArgs A) {
-    constexpr int R1 = croft_plane_r1(NY), R2 = NY / R1;
+    constexpr int R1 = croft_plane_r1y(NY), R2 = NY / R1;
+    using C = typename TwoComplex<croft_plane_axis(NY, false).packed != 0>::type;
     constexpr unsigned DIV_NY = (unsigned)((0x100000000ull + NY - 1) / NY);
-    extern __shared__ __align__(16) float2 plane_tile[];
+    extern __shared__ __align__(16) float2 plane_raw[];
+    C* plane_tile = reinterpret_cast<C*>(plane_raw);
     pdl_allow_dependents();
     const int nz = A.nz, ld = A.ld;
     unsigned short* slot = reinterpret_cast<unsigned short*>(plane_tile + NY * ld);
@@ -91,8 +96,8 @@ __global__ void __launch_bounds__(1024) croft_plane_pass_kernel(const __grid_con
     __syncthreads();
     for (int i = threadIdx.x; i < nz * R2; i += blockDim.x) {
         const int b = (int)__umulhi((unsigned)i, A.div_nz), s = slot[i - b * nz];
-        float2* d = plane_tile + b * ld + s;
-        float2 v[R1];
+        C* d = plane_tile + b * ld + s;
+        C v[R1];
 #pragma unroll
         for (int j = 0; j < R1; ++j) v[j] = d[j * R2 * ld];
         dft<R1>(v);
@@ -102,17 +107,17 @@ __global__ void __launch_bounds__(1024) croft_plane_pass_kernel(const __grid_con
     __syncthreads();
     for (int i = threadIdx.x; i < nz * R1; i += blockDim.x) {
         const int k = (int)__umulhi((unsigned)i, A.div_nz), kz = i - k * nz;
-        const float2* d = plane_tile + (k * R2) * ld + slot[kz];
-        float2 v[R2];
+        const C* d = plane_tile + (k * R2) * ld + slot[kz];
+        C v[R2];
 #pragma unroll
         for (int j = 0; j < R2; ++j) v[j] = d[j * ld];
 #pragma unroll
-        for (int j = 1; j < R2; ++j) v[j] = cmul(v[j], A.tw_y[j * R1 + k]);
+        for (int j = 1; j < R2; ++j) v[j] = cmul(v[j], reinterpret_cast<const C*>(A.tw_y)[j * R1 + k]);
         dft<R2>(v);
-        float2* o = out + k * nz + kz;
+        C* o = reinterpret_cast<C*>(out) + k * nz + kz;
 #pragma unroll
         for (int j = 0; j < R2; ++j) {
-            v[j].y *= A.isign;
+            conj_if(v[j], A.isign);
             o[j * R1 * nz] = v[j];
         }
     }

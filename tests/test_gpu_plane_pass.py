@@ -35,11 +35,20 @@ def _check(croft, shape):
         assert torch.equal(torch.view_as_real(out), torch.view_as_real(c))
         croft.croft_plan_set_timing(p.handle, True)  # an axis at a time
         t = p.forward(d)
+        u = p.backward(d)
         n = len(croft.croft_plan_pass_times(p.handle))
         assert n == croft.croft_plan_num_launches(p.handle) == (3 if shape[0] > 1 else 2)
-    ref = oracle.forward(x)
-    assert oracle.rel_l2(out.cpu().numpy(), ref) <= tol, shape
-    assert oracle.rel_l2(t.cpu().numpy(), ref) <= tol, shape
+        croft.croft_plan_set_timing(p.handle, False)
+        a = torch.empty_like(d)
+        croft.croft_exec_axes(p.handle, d, a, 7, -1)
+    with croft.BatchPlan([shape], mode=croft.CROFT_BATCH_GROUPED) as p:
+        (g,) = p.forward([d])
+        torch.cuda.synchronize()
+    # the passes' own splits and sums: the same bits axis by axis, timed, and in a batch
+    for other in (t, a, g):
+        assert torch.equal(torch.view_as_real(out), torch.view_as_real(other)), shape
+    assert torch.equal(torch.view_as_real(b), torch.view_as_real(u)), shape
+    assert oracle.rel_l2(out.cpu().numpy(), oracle.forward(x)) <= tol, shape
     assert oracle.rel_l2(b.cpu().numpy(), oracle.backward(x)) <= tol, shape
 
 

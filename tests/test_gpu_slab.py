@@ -81,12 +81,16 @@ def test_exec_axes_subsets_match_the_oracle(croft_lib):
                     if mask & (1 << ax):
                         ref = oracle.dft_along_axis(ref, ax, direction)
                 assert oracle.rel_l2(out.cpu().numpy(), ref) <= tol(x.shape), (mask, direction)
-        # in place, and the same bits as exec_forward for all three axes
-        y = p.forward(d)
-        z = d.clone()
-        croft_lib.croft_exec_axes(p.handle, z, z, 7, -1)
-        torch.cuda.synchronize()
-        assert torch.equal(y.view(torch.float32), z.view(torch.float32))
+    # in place, and the same bits as exec_forward for all three axes (the second grid's z and y axes run as one pass there)
+    for shape in (x.shape, (24, 48, 36)):
+        d = torch.from_numpy(S.white_noise(shape, 5)).cuda()
+        with croft_lib.Plan(*shape) as p:
+            assert ("z+y in one pass" in p.describe()) == (shape[1] == 48)
+            y = p.forward(d)
+            z = d.clone()
+            croft_lib.croft_exec_axes(p.handle, z, z, 7, -1)
+            torch.cuda.synchronize()
+        assert torch.equal(y.view(torch.float32), z.view(torch.float32)), shape
     # schedules with more than one launch per axis refuse (256 x 128 x 128: two 16 MiB slabs)
     with croft_lib.Plan(256, 128, 128, schedule=croft_lib.CROFT_SCHEDULE_SLAB_L2) as p:
         assert croft_lib.croft_plan_num_launches(p.handle) > 3
