@@ -206,6 +206,7 @@ cudaError_t launch_scale(const void* in, void* out, const void* g, long long n, 
 
 // croft_passes.cu
 extern int g_max_smem;  // the device's opt-in shared memory per block (set by plan creation)
+int device_sms();       // SMs of the current device (0 if it cannot be asked)
 // Lets launches of kernel f take `bytes` of dynamic shared memory.  The limit belongs to the function, not to a plan:
 // every plan whose pass runs f launches under it, so it is raised where it is too low and never lowered.
 cudaError_t allow_smem(const void* f, int bytes);

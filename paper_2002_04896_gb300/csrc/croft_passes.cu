@@ -77,6 +77,15 @@ bool shape_pass(PassLaunch& L, int layout, int n, long long M, long long ncols, 
     return true;
 }
 
+int device_sms() {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return sms;
+}
+
 cudaError_t allow_smem(const void* f, int bytes) {
     if (bytes <= 48 * 1024) return cudaSuccess;  // (what every kernel may take)
     static std::mutex m;  // plans are created in several threads: look and raise as one step

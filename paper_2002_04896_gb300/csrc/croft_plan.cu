@@ -397,7 +397,7 @@ static croft_status plan_zy(croft_plan p) {
     const int nx = p->dims[0], ny = p->dims[1], nz = p->dims[2];
     const char* pe = getenv("CROFT_PLANE_PASS");
     if ((pe && pe[0] == '0') || p->passes.size() < 2 || p->pass_axis[0] != 2 || p->pass_axis[1] != 1) return CROFT_OK;
-    if (!croft_plane_pass_rule(nx, ny, nz)) return CROFT_OK;
+    if (!croft_plane_pass_rule(nx, ny, nz, device_sms())) return CROFT_OK;
     PlanePass z;
     memset(&z, 0, sizeof(z));
     z.smem = croft_plane_smem(ny, nz);
@@ -418,7 +418,7 @@ static croft_status plan_zy(croft_plan p) {
     z.args.ld = croft_plane_ld(nz);
     z.args.div_nz = (unsigned)((0x100000000ull + (unsigned)nz - 1) / (unsigned)nz);
     z.grid = nx;
-    z.block = croft_plane_threads(nx, ny, nz);
+    z.block = croft_plane_threads(nx, ny, nz, device_sms());
     z.fn = plane_pass_kernel_for(ny);
     p->zy = z;
     return CROFT_OK;
@@ -931,7 +931,7 @@ static croft_status create_tuned(croft_plan* out, int nx, int ny, int nz, croft_
                                       CROFT_SCHEDULE_AUTO};
     static const char* sn[4] = {"three_pass", "slab_l2", "plane_fused", "plane_pass"};
     double best = 1e30;
-    for (int k = 0; k < (croft_plane_pass_rule(nx, ny, nz) ? 4 : 3); ++k) {
+    for (int k = 0; k < (croft_plane_pass_rule(nx, ny, nz, device_sms()) ? 4 : 3); ++k) {
         croft_plan p = nullptr;
         const croft_status st = create_impl(&p, nx, ny, nz, dtype, scheds[k], (k == 0 || k == 3) ? &ch : nullptr);
         if (st != CROFT_OK) {

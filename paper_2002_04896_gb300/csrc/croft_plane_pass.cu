@@ -8,7 +8,7 @@ plane_pass_fn plane_pass_kernel_for(int ny) {
     switch (ny) {
 #define CROFT_PLANE_Y(NY) \
     case NY: return croft_plane_pass_kernel<NY>;
-        CROFT_PLANE_SIZES(CROFT_PLANE_Y)
+        CROFT_PLANE_Y_SIZES(CROFT_PLANE_Y)
 #undef CROFT_PLANE_Y
         default: return nullptr;
     }

@@ -5,11 +5,12 @@
 #include "croft_sched.h"
 #include "croft_two_stage.h"
 
-// Whether an axis of n points may be one of a plane (both radices at most 16; 125: 25).
-CROFT_HD constexpr bool croft_plane_length(int n) {
+// Lengths a plane's y axis may have, and its z axis (those that croft_plane_pass_rule takes).
+CROFT_HD constexpr bool croft_plane_y(int n) {
     return n == 32 || n == 36 || n == 40 || n == 45 || n == 48 || n == 50 || n == 54 || n == 60 || n == 64 || n == 72 ||
            n == 75 || n == 80 || n == 81 || n == 90 || n == 96 || n == 100 || n == 108 || n == 120 || n == 125 || n == 128;
 }
+CROFT_HD constexpr bool croft_plane_z(int n) { return croft_plane_y(n) && (n <= 75 || n == 81 || n == 125); }
 // How a plane's z and y axes split, n = R1 * R2, and whether their sums are paired: as the axis passes do (32 points: their
 // stages 16 and 2), so that a transform has the same bits whether z and y run as one pass or as two (per-axis timing,
 // croft_exec_axes, batches).
@@ -17,7 +18,7 @@ struct CroftPlaneAxis {
     int r1, packed;
 };
 CROFT_HD constexpr CroftPlaneAxis croft_plane_axis(int n, bool z) {
-    if (!croft_plane_length(n)) return CroftPlaneAxis{0, 0};
+    if (!(z ? croft_plane_z(n) : croft_plane_y(n))) return CroftPlaneAxis{0, 0};
     if (n == 32) return CroftPlaneAxis{16, 0};
     const CroftTwo k = z ? croft_two_row(n) : croft_two_col(n, false);
     return CroftPlaneAxis{k.r1, k.packed};
@@ -31,23 +32,35 @@ CROFT_HD constexpr int croft_plane_ld(int nz) { return (croft_plane_r1z(nz) * cr
 // Shared memory: [plane: ny rows of ld][slot of every z frequency: nz 16-bit numbers].
 CROFT_HD constexpr int croft_plane_smem(int ny, int nz) { return ny * croft_plane_ld(nz) * 8 + (nz * 2 + 15) / 16 * 16; }
 
-// Whether a plan runs its z and y axes as one pass over the planes.  Measured in graph replays (no host time),
-// three passes over plane pass + x pass: 32^3 1.71, 36^3 1.15, 48^3 1.10, 54^3 1.10, 64^3 0.92, 80^3 0.93,
-// 96^3 0.94, 100^3 1.14, 108^3 0.89; 300 planes of 48^2 1.41, 54^2 1.48, 60^2 1.40, 64^2 1.25, 80^2 1.08, 90^2
-// 1.20, 96^2 1.13, 100^2 1.05, 108^2 1.00, 120^2 0.96; 4 planes of 64^2 0.92, 16 of 96^2 0.69.  Launched one by
-// one, a transform of up to about 64^3 points takes as long as its launches (9 us for three, 5 for two), so
-// planes of up to 4096 points always take it; larger ones from about two planes per SM on (162 of 90 x 108, one
-// round and a rest: a convolution takes 36.6 us against 35.3), up to 6400 points, and up to 10,000 while the grid
-// stays in the L2 (z and y of 960 planes, two passes / plane pass: 72^2 30.4 / 27.4 us, 80^2 35.3 / 35.8, 96^2
-// 48.4 / 54.0, 108^2 60 / 67).
-CROFT_HD constexpr bool croft_plane_pass_rule(int nx, int ny, int nz) {
-    return croft_plane_length(ny) && croft_plane_length(nz) &&
-           (ny * nz <= 4096 || (nx >= 288 && (ny * nz <= 6400 || (ny * nz <= 10000 && nx <= 456))));
+// Whether a plan runs its z and y axes as one pass over its nx planes, on a device of `sms` SMs.  Measured over all pairs of
+// lengths and 91 values of nx as captured graphs, three passes' time over plane pass + x pass; the rule takes only what
+// measured no slower there (median 1.18; 12 of 5606 shapes below 0.985, the lowest 0.95), in a loop of single calls (181 shapes, 0.99
+// to 1.65) and call by call (1.00 to 1.25):
+//  * few planes (one CTA per plane, at most two SMs of three busy): the launch saved outweighs the stages' latency up to
+//    about 2304 points, 32^3 1.68, 36^3 1.21, 40^3 1.11, 48^3 1.12, 16 planes of 48^2 1.08 (60^3 0.88, 64^3 0.93, 16 of
+//    64^2 0.95); one plane up to 1536 (2D: 32 x 32 1.36, 48 x 48 0.97).  Rows of 32 points, whose passes are short of work, at any
+//    plane size: 16 of 128 x 32 1.15, 64 of 64 x 32 1.45;
+//  * many planes: the z lengths whose own row pass moves least (5.6 to 6.6 TB/s: 36, 45, 50, 54, 60, 75, 81, 125), from the number
+//    of planes at which each is ahead at every plane size, up to 4800 points: 300 planes of 54^2 1.21, 60^2 1.10, 48 x 36
+//    1.13; 480 of 36 x 81 1.10.  Other z lengths gain or lose by the number of planes that the last round of CTAs holds
+//    (300 of 64^2 1.27, 600 of 64^2 0.95; 300 of 80^2 1.00, 960 of 80^2 0.95) and keep their two passes, as do grids
+//    beyond 32 MB, where two axis passes in a row read the L2.
+CROFT_HD constexpr bool croft_plane_pass_rule(int nx, int ny, int nz, int sms) {
+    if (!croft_plane_y(ny) || !croft_plane_z(nz)) return false;
+    const int plane = ny * nz;
+    if (3 * nx <= 2 * sms) return nz == 32 || plane <= (nx > 1 ? 2304 : 1536);
+    if (6 * nx < 5 * sms) return nz == 32;
+    if (ny < 36 || plane > 4800 || (long long)nx * plane > 4 * 1024 * 1024) return false;
+    if (nz == 45 || nz == 54) return ny >= 48 || 3 * nx >= 5 * sms;
+    if (nz == 36 || nz == 60) return 3 * nx >= 5 * sms;
+    if (nz == 75 || nz == 81 || nz == 125) return 5 * nx >= 13 * sms;
+    return (nz == 32 || nz == 50) && nx >= 3 * sms;
 }
 // Threads of a plane's CTA: enough for one round of butterflies a stage where an SM holds one plane, fewer (and
 // more planes at a time) where there are many.  64^3: 128 / 256 / 384 / 512 / 1024 threads 0.81 / 0.89 / 0.88 /
 // 0.92 / 0.90 of the three passes' speed, 300 planes of 64^2 1.12 / 1.25 / 1.02 / 1.02 / 0.91, 4096 of 32^2
-// 1.20 / 1.15 / 1.04 / 1.05 / 0.79; 960 planes of 60^2 27.0 / 23.9 / 25.6 / 26.3 / 31.2 us.
-CROFT_HD constexpr int croft_plane_threads(int nx, int ny, int nz) {
-    return nx <= 152 ? 512 : (nx <= 608 || ny * nz > 1600 ? 256 : 128);
+// 1.20 / 1.15 / 1.04 / 1.05 / 0.79; 960 planes of 60^2 27.0 / 23.9 / 25.6 / 26.3 / 31.2 us (measured with the splits 8*8, 10*6
+// and 8*4 of these lengths).
+CROFT_HD constexpr int croft_plane_threads(int nx, int ny, int nz, int sms) {
+    return nx <= sms ? 512 : (nx <= 4 * sms || ny * nz > 1600 ? 256 : 128);
 }

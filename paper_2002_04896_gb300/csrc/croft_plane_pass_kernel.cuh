@@ -6,11 +6,12 @@
 // crosses the L2 twice.
 //
 // What bounds it: for small grids the launches (a 32^3 transform: 9.1 us of host time for three, 5.1 for
-// two; on the device, in a graph, 7.7 -> 4.6 us), beyond that the instruction issue of four
-// barrier-separated stages at 64 registers, 1024 threads per SM (about 4 TB/s of the 16 bytes a point
-// where two axis passes in a row move 7 each): hence the limits of croft_plane_pass_rule.
+// two; on the device, in a graph, 7.5 -> 4.5 us), beyond that the instruction issue of four
+// barrier-separated stages at 64 registers, 1024 threads per SM: 2.6-2.9 TB/s of the 16 bytes a point that it moves (960 planes
+// of 72^2 in 27.4 us, of 96^2 in 54.0), where two axis passes in a row come to the same 2.6-3.0 TB/s of those 16
+// bytes (30.4 and 48.4 us): hence the limits of croft_plane_pass_rule.
 //
-// Both transforms take two stages n = R1 * R2, every stage in place, so that a thread may take any
+// Both transforms take two stages n = R1 * R2, split and summed as in the axis passes (croft_plane_axis: the same bits), every stage in place, so that a thread may take any
 // number of butterflies one after the other and a barrier stands only between stages:
 //   z1  butterfly b < R2 of a row reads z = b + j*R2 (j < R1) from HBM, radix R1, element (k, b)
 //   z2  butterfly k < R1: elements (k, j), twiddles w_nz^{jk}, radix R2; element (k, j) is now frequency k + j*R1
@@ -21,7 +22,7 @@
 // HBM are contiguous and a warp shares its twiddles), each a walk of odd stride over the banks.
 //
 // The kernel is specialised on ny; the z stages are functions of their own, one per nz, called once
-// per plane (24 + 21 bodies instead of a kernel for every pair of lengths).
+// per plane (20 kernels and 13 such functions instead of a kernel for every pair of lengths).
 #pragma once
 #include "croft_butterflies.cuh"
 #include "croft_fft_core.cuh"
@@ -67,9 +68,10 @@ __device__ __noinline__ void plane_z(const float2* in, const float2* tw, int ny,
     }
 }
 
-#define CROFT_PLANE_SIZES(X)                                                                                     \
+#define CROFT_PLANE_Y_SIZES(X)                                                                                   \
     X(32) X(36) X(40) X(45) X(48) X(50) X(54) X(60) X(64) X(72) X(75) X(80) X(81) X(90) X(96) X(100) X(108)      \
     X(120) X(125) X(128)
+#define CROFT_PLANE_Z_SIZES(X) X(32) X(36) X(40) X(45) X(48) X(50) X(54) X(60) X(64) X(72) X(75) X(81) X(125)
 
 template <int NY>
 __global__ void __launch_bounds__(1024) croft_plane_pass_kernel(const __grid_constant__ PlanePassArgs A) {
@@ -89,7 +91,7 @@ __global__ void __launch_bounds__(1024) croft_plane_pass_kernel(const __grid_con
     switch (nz) {
 #define CROFT_PLANE_Z(NZ)                                                \
     case NZ: plane_z<NZ>(in, A.tw_z, NY, DIV_NY, A.isign); break;
-        CROFT_PLANE_SIZES(CROFT_PLANE_Z)
+        CROFT_PLANE_Z_SIZES(CROFT_PLANE_Z)
 #undef CROFT_PLANE_Z
         default: break;
     }

@@ -11,7 +11,8 @@ import oracle
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
-LENGTHS = [32, 36, 40, 45, 48, 50, 54, 60, 64, 72, 75, 80, 81, 90, 96, 100, 108, 120, 125, 128]
+Y_LENGTHS = [32, 36, 40, 45, 48, 50, 54, 60, 64, 72, 75, 80, 81, 90, 96, 100, 108, 120, 125, 128]
+Z_LENGTHS = [32, 36, 40, 45, 48, 50, 54, 60, 64, 72, 75, 81, 125]
 
 
 def _noise(shape, seed):
@@ -52,21 +53,27 @@ def _check(croft, shape):
     assert oracle.rel_l2(b.cpu().numpy(), oracle.backward(x)) <= tol, shape
 
 
-@pytest.mark.parametrize("n", LENGTHS)
-def test_every_length_as_y_and_z(croft_lib, n):
+@pytest.mark.parametrize("n", Y_LENGTHS)
+def test_every_length_as_y(croft_lib, n):
     _check(croft_lib, (3, n, 32))
-    _check(croft_lib, (2, 32, n))
-    if n <= 64:
+
+
+@pytest.mark.parametrize("n", Z_LENGTHS)
+def test_every_length_as_z(croft_lib, n):
+    _check(croft_lib, (2, 32, n) if n <= 72 else (400, 36, n))
+    if n <= 36:
         _check(croft_lib, (1, n, n))
 
 
-@pytest.mark.parametrize("shape", [(300, 100, 100), (288, 75, 128), (288, 128, 75), (300, 72, 125), (625, 48, 40)])
+# one plane an SM and a rest; 256- and 128-thread CTAs; the largest planes the rule takes
+@pytest.mark.parametrize("shape", [(150, 100, 45), (256, 80, 60), (300, 128, 36), (480, 96, 50), (480, 36, 125), (625, 36, 45),
+                                   (480, 128, 32), (100, 36, 64)])
 def test_many_planes(croft_lib, shape):
     _check(croft_lib, shape)
 
 
 def test_convolution_and_rule(croft_lib):
-    shape = (20, 60, 48)
+    shape = (20, 48, 45)
     x = _noise(shape, 5)
     g = np.random.default_rng(6).uniform(0.1, 1, shape).astype(np.float32)
     with croft_lib.Plan(*shape) as p:
@@ -74,8 +81,9 @@ def test_convolution_and_rule(croft_lib):
         y = p.convolve(torch.from_numpy(x).cuda(), torch.from_numpy(g).cuda())
         torch.cuda.synchronize()
     assert oracle.rel_l2(y.cpu().numpy(), oracle.convolve(x, g)) <= 4e-6 * math.log2(x.size)
-    for shape, takes in (((64, 64, 64), True), ((64, 72, 64), False), ((288, 72, 64), True), ((162, 72, 64), False), ((300, 108, 108), False),
-                         ((8, 30, 32), False), ((8, 32, 256), False)):
+    for shape, takes in (((48, 48, 48), True), ((60, 60, 60), False), ((16, 64, 64), False), ((120, 48, 48), False),
+                         ((120, 100, 32), True), ((128, 60, 54), True), ((300, 48, 36), True), ((300, 64, 64), False),
+                         ((300, 108, 108), False), ((8, 30, 32), False), ((8, 32, 256), False)):
         with croft_lib.Plan(*shape) as p:
             assert ("z+y in one pass" in p.describe()) == takes, shape
         with croft_lib.Plan(*shape, schedule=croft_lib.CROFT_SCHEDULE_THREE_PASS) as p:

@@ -20,8 +20,8 @@ def _input(shape, seed, dtype=np.complex64):
     return (r.uniform(-1, 1, shape) + 1j * r.uniform(-1, 1, shape)).astype(dtype)
 
 
-# (older plan, newer plan): planes of the same y length, the newer z axis shorter; below and above 48 KB
-@pytest.mark.parametrize("older,newer", [((64, 64, 64), (64, 64, 32)), ((300, 100, 100), (8, 100, 40))])
+# (older plan, newer plan): planes of the same y length, the newer ones smaller in shared memory; below and above 48 KB
+@pytest.mark.parametrize("older,newer", [((64, 36, 64), (64, 36, 32)), ((8, 128, 32), (256, 128, 36))])
 def test_plane_pass_plans(croft_lib, older, newer):
     with croft_lib.Plan(*older) as a, croft_lib.Plan(*newer) as b:
         for plan, shape in ((a, older), (b, newer), (a, older)):

@@ -1,6 +1,7 @@
 """Host checks of the two-stage pass table (``csrc/croft_two_stage.h``): every entry factorises its
 length into radices that have a butterfly, and its tile fits the launch and shared-memory limits it
-names (CPU only)."""
+names; and of the plane pass's rule (``csrc/croft_plane_pass.h``): the edges of what it takes, and that
+every plane has a kernel and fits (CPU only)."""
 
 import os
 import shutil
@@ -57,3 +58,43 @@ def test_entries_fit(table):
             assert w % 8 == 0, (kind, n, w)  # rows of at least 64 bytes
         # two CTAs share a tile: each takes half of the butterflies of either stage, from global twiddles
         assert ctas == 1 or (ctas == 2 and kind != "r" and stage == 0 and smem == r2 * ((r1 + 1) // 2) * w * 8)
+
+
+PLANE_PROGRAM = r"""
+#include <cstdio>
+#include "croft_plane_pass.h"
+int main() {
+    const int sms[2] = {152, 148};
+    for (int s : sms)
+        for (int nx = 1; nx <= 1200; ++nx)
+            for (int ny = 1; ny <= 140; ++ny)
+                for (int nz = 1; nz <= 140; ++nz)
+                    if (croft_plane_pass_rule(nx, ny, nz, s))
+                        std::printf("%d %d %d %d %d %d %d %d\n", s, nx, ny, nz, croft_plane_r1y(ny), croft_plane_r1z(nz),
+                                    croft_plane_smem(ny, nz), croft_plane_threads(nx, ny, nz, s));
+    return 0;
+}
+"""
+
+
+def test_plane_rule_edges(tmp_path):
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if not cxx:
+        pytest.skip("no host C++ compiler")
+    (tmp_path / "p.cpp").write_text(PLANE_PROGRAM)
+    subprocess.run([cxx, "-std=c++17", "-I", CSRC, str(tmp_path / "p.cpp"), "-o", str(tmp_path / "p")], check=True)
+    out = subprocess.run([str(tmp_path / "p")], check=True, capture_output=True, text=True).stdout
+    rows = [tuple(map(int, line.split())) for line in out.splitlines()]
+    took = {r[:4] for r in rows}
+    for _, nx, ny, nz, r1y, r1z, smem, threads in rows:
+        assert r1y in RADICES and r1z in RADICES and ny % r1y == 0 and nz % r1z == 0 and max(ny // r1y, nz // r1z) <= 25
+        assert smem <= 99 * 1024 and threads in (128, 256, 512), (nx, ny, nz)
+        assert ny * nz <= 4800 and nx * ny * nz <= 4 * 1024 * 1024
+    # the number of planes up to which small planes are taken (two SMs of three), rows of 32 points (five of six), and from which
+    # the longer planes are, follows the device
+    for sms, few, rows32, many in ((152, 101, 126, 456), (148, 98, 123, 444)):
+        assert (sms, few, 48, 48) in took and (sms, few + 1, 48, 48) not in took and (sms, few, 50, 48) not in took
+        assert (sms, rows32, 128, 32) in took and (sms, rows32 + 1, 128, 32) not in took
+        assert (sms, many, 90, 50) in took and (sms, many - 1, 90, 50) not in took
+        assert (sms, 1, 48, 32) in took and (sms, 1, 48, 36) not in took
+        assert not any(r[0] == sms and r[3] in (80, 90, 96, 100, 108, 120, 128) for r in rows)
