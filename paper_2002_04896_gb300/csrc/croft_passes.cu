@@ -43,7 +43,7 @@ bool shape_pass(PassLaunch& L, int layout, int n, long long M, long long ncols, 
         int W = (256 + T - 1) / T;
         if (W < 1) W = 1;
         while (W > 1 && (W * T > max_threads || (A.tw_pad + (long long)W * ld) * es > smem_cap)) --W;
-        if (f64 && croft_half_tiles64(ncols, W)) W /= 2;
+        if (f64 && croft_half_tiles64(ncols, W, device_sms())) W /= 2;
         if ((long long)W > ncols && !tc) W = (int)ncols;  // (tensor-core tiles keep whole 128-row groups)
         A.W = W;
         L.smem = (int)((A.tw_pad + (long long)W * ld) * es);
@@ -55,7 +55,7 @@ bool shape_pass(PassLaunch& L, int layout, int n, long long M, long long ncols, 
             W = croft_col_width_at(n, (int)es, M * es);  // a width the kernels are built for
         }
         if (want_w >= 1 && !tc) W = want_w;
-        else if (f64 && croft_col_half64(n) * 2 == W && croft_half_tiles64(ncols, W)) W /= 2;
+        else if (f64 && croft_col_half64(n) * 2 == W && croft_half_tiles64(ncols, W, device_sms())) W /= 2;
         while (W > 1 && (W * T > max_threads || (A.tw_pad + (long long)n * W) * es > smem_cap)) W /= 2;
         A.W = W;
         L.smem = (int)((A.tw_pad + (long long)n * W) * es);
@@ -216,9 +216,7 @@ bool shape_ring(PassLaunch& L, int n, long long M, long long ncols) {
         cudaGetLastError();
         return false;
     }
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = device_sms();
     L.grid = (int)(R.ntiles < (long long)sms ? R.ntiles : (long long)sms);
     return L.grid > 0 && tensor_map_encoder() != nullptr;
 }

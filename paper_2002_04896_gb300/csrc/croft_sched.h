@@ -212,12 +212,11 @@ CROFT_HD constexpr int croft_col_half64(int n) {
 
 // Whether a complex128 pass over ncols pencils takes half tiles instead of tiles of w pencils.  These passes
 // keep the FP64 pipes busy, so a pass lasts as long as the SM with the most pencils, and the hardware hands out
-// whole tiles: half tiles where their rounds come to fewer pencils on the fullest of 152 SMs.  Per transform, tiles / half
-// tiles: 16^3 43 / 25 us, 64^3 62 / 37, 60x96x120 135 / 104, 96x128x120 215 / 197, 128^3 266 / 234; where both
+// whole tiles: half tiles where their rounds come to fewer pencils on the fullest of the device's SMs (152 here).  Per
+// transform, tiles / half tiles: 16^3 43 / 25 us, 64^3 62 / 37, 60x96x120 135 / 104, 96x128x120 215 / 197, 128^3 266 / 234; where both
 // come to the same, 120^3 226 / 231, 96^3 119 / 116, 256^3 2025 / 2023 us.
-CROFT_HD constexpr bool croft_half_tiles64(long long ncols, int w) {
-    const long long sms = 152;
-    if (w % 2) return false;
+CROFT_HD constexpr bool croft_half_tiles64(long long ncols, int w, int sms) {
+    if (w % 2 || sms < 1) return false;
     const long long full = ((ncols + w - 1) / w + sms - 1) / sms * w;
     const long long half = ((ncols + w / 2 - 1) / (w / 2) + sms - 1) / sms * (w / 2);
     return half < full;

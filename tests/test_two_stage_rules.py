@@ -98,3 +98,28 @@ def test_plane_rule_edges(tmp_path):
         assert (sms, many, 90, 50) in took and (sms, many - 1, 90, 50) not in took
         assert (sms, 1, 48, 32) in took and (sms, 1, 48, 36) not in took
         assert not any(r[0] == sms and r[3] in (80, 90, 96, 100, 108, 120, 128) for r in rows)
+
+
+def test_half_tiles_follow_the_sm_count(tmp_path):
+    """complex128 half tiles: taken exactly where the fullest of the device's SMs then has fewer pencils."""
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if not cxx:
+        pytest.skip("no host C++ compiler")
+    (tmp_path / "h.cpp").write_text("""
+#include <cstdio>
+#include "croft_sched.h"
+int main() {
+    const int sms[3] = {152, 148, 1};
+    for (int s : sms)
+        for (int n = 1; n <= 20000; n += 37) std::printf("%d %d %d\\n", s, n, (int)croft_half_tiles64(n, 16, s));
+    std::printf("0 0 %d\\n", (int)croft_half_tiles64(100, 16, 0) + (int)croft_half_tiles64(100, 15, 152));
+    return 0;
+}
+""")
+    subprocess.run([cxx, "-std=c++17", "-I", CSRC, str(tmp_path / "h.cpp"), "-o", str(tmp_path / "h")], check=True)
+    out = subprocess.run([str(tmp_path / "h")], check=True, capture_output=True, text=True).stdout
+    rows = [tuple(map(int, line.split())) for line in out.splitlines()]
+    assert rows[-1] == (0, 0, 0)
+    for s, n, half in rows[:-1]:
+        assert half == (-(-(-(-n // 8)) // s) * 8 < -(-(-(-n // 16)) // s) * 16), (s, n)
+    assert [r[2] for r in rows if r[0] == 152] != [r[2] for r in rows if r[0] == 148]
