@@ -109,6 +109,31 @@ def test_pme_batch_96_grouped_matches_single_grid_plans_bitwise(croft_lib, pme_b
         assert oracle.rel_l2(a[g].cpu().numpy(), oracle.forward(x)) <= tol(x.shape)
 
 
+@pytest.mark.parametrize("count", [32, 33, 70])
+def test_grouped_batch_of_many_grids_of_one_length(croft_lib, count):
+    """A launch holds 32 grids of one length: full, one over, and three launches per pass (y and z axes of 36 points)."""
+    dims = [(2 + g % 7, 36, 36) for g in range(count)]
+    dims = [(d[0] + (d[0] == 7), 36, 36) for d in dims]  # (7 is no supported length)
+    rng = np.random.default_rng(count)
+    xs = [(rng.uniform(-1, 1, d) + 1j * rng.uniform(-1, 1, d)).astype(np.complex64) for d in dims]
+    ins = [torch.from_numpy(x).cuda() for x in xs]
+    with croft_lib.BatchPlan(dims, mode=croft_lib.CROFT_BATCH_GROUPED) as bp:
+        per_pass = -(-count // 32)
+        x_lengths = [d[0] for d in dims]
+        x_launches = sum(-(-x_lengths.count(n) // 32) for n in set(x_lengths))
+        assert croft_lib.croft_plan_num_launches(bp.handle) == 2 * per_pass + x_launches
+        f = bp.forward(ins)
+        b = bp.backward(ins)
+        c = [t.clone() for t in ins]
+        bp.forward(c, c)  # in place
+        torch.cuda.synchronize()
+    for g, x in enumerate(xs):
+        t = tol(x.shape)
+        assert oracle.rel_l2(f[g].cpu().numpy(), oracle.forward(x)) <= t, (count, g)
+        assert oracle.rel_l2(b[g].cpu().numpy(), oracle.backward(x)) <= t, (count, g)
+        assert torch.equal(f[g].view(torch.int32), c[g].view(torch.int32)), (count, g)
+
+
 def test_autotune_chooses_and_caches(croft_lib, pme_batch, tmp_path, monkeypatch):
     dims, _ = pme_batch
     cache = tmp_path / "tune.txt"

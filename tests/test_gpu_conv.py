@@ -226,14 +226,20 @@ def test_full_size_properties(croft_lib, dev, name):
 
 
 @pytest.mark.parametrize("n", [320, 512])
-def test_fused_axis_on_the_radix16_first_split(croft_lib, dev, n):
-    """Axes whose passes take the radix-16-first split by the rules (320; 512 at short strides)
-    keep the fused convolution: it runs its own schedule on a twiddle table of its own."""
+@pytest.mark.parametrize("general", [False, True])
+def test_fused_axis_whose_pass_splits_differently(croft_lib, dev, n, general, monkeypatch):
+    """Axes whose general passes take the radix-16-first split by the rules (320; 512 at short strides) keep the
+    fused convolution, which runs two stages of its own whatever the axis's pass runs."""
+    if general:
+        monkeypatch.setenv("CROFT_TWO_STAGE", "0")
     shape = (n, 2, 3)
     with croft_lib.Plan(*shape) as p:
         d = p.describe()
     x_pass = d[d.index("x:"):].split(" | ")[0]
-    assert ("radix=16x5x4" if n == 320 else "radix=16x8x4") in x_pass, d
+    if general:
+        assert ("radix=16x5x4" if n == 320 else "radix=16x8x4") in x_pass and "->" not in x_pass, d
+    else:
+        assert ("-> two-stage 20x16" if n == 320 else "-> two-stage 32x16") in x_pass, d
     assert "fwd*G*bwd fused" in d, d
     x, g = _inputs(shape, 400 + n)
     y, _ = conv_gpu(croft_lib, x, g)

@@ -70,26 +70,36 @@ def _pass_desc(desc, axis):
     return part.split(" | ")[0]
 
 
+@pytest.fixture(params=["general", "two-stage"])
+def kernels(request, monkeypatch):
+    """Which kernels the passes run: the general ones (two-stage kernels off) or the default plan's."""
+    if request.param == "general":
+        monkeypatch.setenv("CROFT_TWO_STAGE", "0")
+    return request.param
+
+
 @pytest.mark.parametrize("n", LONG_PENCIL_SIZES)
-def test_long_pencil_x_pass_over_wide_stride(croft_lib, dev, n):
+def test_long_pencil_x_pass_over_wide_stride(croft_lib, dev, n, kernels):
     """A length of 32-thread pencils as the x axis with its elements 18 KB apart takes the
-    16-column tile (the y pass of the length-n axis above, 40 bytes apart, the 8-column one);
+    16-column tile (the general kernel's y pass of the length-n axis above, 40 bytes apart, the 8-column one);
     2250 columns leave a ragged last tile."""
     rng = np.random.default_rng(1000 + n)
     shape = (n, 45, 50)
     x = (rng.uniform(-1, 1, shape) + 1j * rng.uniform(-1, 1, shape)).astype(np.complex64)
     with croft_lib.Plan(*shape) as p:
-        assert " W=16 " in _pass_desc(p.describe(), "x"), p.describe()
+        d = _pass_desc(p.describe(), "x")
+    assert ("-> two-stage" in d) == (kernels == "two-stage") and " W=16 " in d.split("->")[-1], d
     y = run(croft_lib, x)
     e = oracle.rel_l2(y, oracle.forward(x))
     assert e <= tol(shape), (shape, e)
 
 
 @pytest.mark.parametrize("n", [270, 320, 324, 360, 384, 405, 432, 480])
-def test_24_thread_pencils_where_the_rule_takes_them(croft_lib, dev, n):
-    """The column passes of these lengths run 24 threads per pencil where the rule says so
+def test_24_thread_pencils_where_the_rule_takes_them(croft_lib, dev, n, monkeypatch):
+    """The general column passes of these lengths run 24 threads per pencil where the rule says so
     (8-column y tiles of 192 threads, 16-column x tiles of 384), 32 elsewhere, against the oracle
     with ragged tiles."""
+    monkeypatch.setenv("CROFT_TWO_STAGE", "0")
     rng = np.random.default_rng(2400 + n)
     for shape, axis, narrow in (((3, n, 5), "y", True), ((n, 45, 50), "x", False)):
         x = (rng.uniform(-1, 1, shape) + 1j * rng.uniform(-1, 1, shape)).astype(np.complex64)
@@ -97,18 +107,20 @@ def test_24_thread_pencils_where_the_rule_takes_them(croft_lib, dev, n):
             d = _pass_desc(p.describe(), axis)
         t24 = n in ((324, 360, 405) if narrow else (324, 360, 384, 405))
         want = (" T=24 W=8 block=192 " if narrow else " T=24 W=16 block=384 ") if t24 else " T=32 "
-        assert want in d, (shape, d)
+        assert want in d and "->" not in d, (shape, d)
         y = run(croft_lib, x)
         e = oracle.rel_l2(y, oracle.forward(x))
         assert e <= tol(shape), (shape, e)
 
 
-def test_16_thread_pencils_by_default_for_432_and_480_across_long_strides(croft_lib, dev):
-    """432- and 480-point x passes across 256 KB or more take 16 threads per pencil (16-column,
+def test_16_thread_pencils_by_default_for_432_and_480_across_long_strides(croft_lib, dev, monkeypatch):
+    """432- and 480-point general x passes across 256 KB or more take 16 threads per pencil (16-column,
     256-thread tiles); shorter strides keep 32 (their parity: the tuned-plan tests)."""
+    monkeypatch.setenv("CROFT_TWO_STAGE", "0")
     for n in (432, 480):
         with croft_lib.Plan(n, 128, 256) as p:
-            assert " T=16 W=16 block=256 " in _pass_desc(p.describe(), "x"), p.describe()
+            d = _pass_desc(p.describe(), "x")
+        assert " T=16 W=16 block=256 " in d and "->" not in d, d
         with croft_lib.Plan(n, 64, 64) as p:
             assert " T=32 " in _pass_desc(p.describe(), "x"), p.describe()
 
@@ -120,7 +132,7 @@ def test_column_width_follows_the_stride(croft_lib, dev, monkeypatch):
     monkeypatch.setenv("CROFT_TWO_STAGE", "0")
     with croft_lib.Plan(512, 512, 512) as p:
         d = p.describe()
-    assert " W=8 block=256 " in _pass_desc(d, "y"), d
+    assert " W=8 block=256 " in _pass_desc(d, "y") and "->" not in d, d
     assert "+pair" in _pass_desc(d, "x") and " W=16 block=256 " in _pass_desc(d, "x"), d
     with croft_lib.Plan(512, 128, 128) as p:
         d = p.describe()

@@ -75,6 +75,7 @@ def test_every_tuner_candidate_matches_the_oracle(croft_lib, cache, n):
                 f.write(f"{key} 1 " + " ".join(str(v) for c in ch for v in c) + " forced\n")
             desc = _check(croft_lib, x, ("tuned (cached)",))
             seg = [s for s in desc.split("|") if s.strip().startswith(("x:", "y:", "z:"))][2 - axis]
+            assert "->" not in seg, seg  # a kernel that a choice names is the one that runs
             if kind == 1:
                 assert "+ring" in seg, seg
             elif kind == 2:

@@ -47,7 +47,18 @@ def test_every_length(croft_lib, n):
         _check(x, y, axis, direction)
 
 
-@pytest.mark.parametrize("n", [640, 729, 810, 1024])
+@pytest.mark.parametrize("n", sorted(LENGTHS))
+def test_every_length_with_the_general_kernels(croft_lib, monkeypatch, n):
+    # (they run with CROFT_TWO_STAGE=0; the same ragged shapes)
+    monkeypatch.setenv("CROFT_TWO_STAGE", "0")
+    for shape, axis, direction in (((n, 3, 25), 0, 1), ((2, n, 27), 1, -1), ((5, 3, n), 2, 1)):
+        x, y, desc = _run(croft_lib, shape, axis, direction, n + axis)
+        assert "two-stage" not in desc, desc
+        _check(x, y, axis, direction)
+
+
+# the lengths whose kernels for long strides differ from those for short ones, and two whose do not
+@pytest.mark.parametrize("n", [640, 675, 720, 729, 750, 768, 800, 810, 864, 1024])
 def test_long_strides(croft_lib, n):
     # elements 262,440 bytes apart: the 16-column tile; 32,805 columns, five in the last tile
     x, y, desc = _run(croft_lib, (n, 81, 405), 0, -1, n)
