@@ -95,7 +95,7 @@ croft_status group_state_build(const std::vector<int>& dims, const std::vector<i
                 return CROFT_ERR_UNSUPPORTED_SIZE;
             }
             const bool row = layout == LAYOUT_ROW;
-            const CroftTwo K = row ? croft_two_row(n) : croft_two_col(n, false);
+            const CroftTwo K = croft_two_batch(n, row);
             const std::pair<int, int> key{n, K.r1};
             if (!tw_off.count(key)) {
                 tw_off[key] = (int)(pool.size() / 2);

@@ -31,7 +31,7 @@ cudaError_t launch_batched(const BatchArgs& A, int blocks, int smem, cudaStream_
 // Capacity of the static scratch (held by every GPU that loads the library until exit).
 constexpr int kNaMaxGrids = CROFT_NOALLOC_MAX_GRIDS;
 constexpr int kNaMaxItems = CROFT_NOALLOC_MAX_ITEMS;
-constexpr int kNaMaxTw = 8192;         // float2 slots; all 37 supported lengths <= 128 need < 2500
+constexpr int kNaMaxTw = 8192;         // float2 slots; the 37 supported lengths <= 128, up to two tables each, need < 4000
 constexpr int kNaCounterInts = 1024;   // [0] work counter, [4] status, [8 + 3 g + pass] completion counts
 constexpr size_t kNaCounters = sizeof(int) * kNaCounterInts;
 constexpr size_t kNaGridsOff = kNaCounters;

@@ -29,6 +29,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <map>
 #include <new>
 #include <string>
 #include <vector>
@@ -45,6 +46,7 @@ cudaError_t batched_prepare(int smem);
 int batched_blocks_per_sm(int smem);
 void* batched_kernel_ptr();
 int host_build_twiddles(int n, float* out);  // croft_plan.cu
+void host_build_two_twiddles(int n, int r1, float* out);
 
 struct GroupState;  // croft_batch_group.cu
 croft_status group_state_build(const std::vector<int>& dims, const std::vector<int>& pgrid, GroupState** out);
@@ -112,20 +114,8 @@ croft_status build_batch_tables(const std::vector<int>& dims, const std::vector<
                                 std::vector<BatchGrid>& hgrid, std::vector<BatchItem>& items,
                                 std::vector<float>& pool, int pass_begin[4]) {
     const int G = (int)pgrid.size();
-    std::vector<int> lens;
-    for (int g : pgrid)
-        for (int a = 0; a < 3; ++a) lens.push_back(dims[3 * g + a]);
-    std::sort(lens.begin(), lens.end());
-    lens.erase(std::unique(lens.begin(), lens.end()), lens.end());
     pool.clear();
-    std::vector<int> off(CROFT_BATCH_MAX_N + 1, 0);
-    for (int n : lens) {
-        if (n > CROFT_BATCH_MAX_N) return CROFT_ERR_UNSUPPORTED_SIZE;
-        off[n] = (int)(pool.size() / 2);
-        std::vector<float> t(2 * (size_t)n + 2, 0.f);
-        if (n > 1 && host_build_twiddles(n, t.data()) != n - 1) return CROFT_ERR_UNSUPPORTED_SIZE;
-        pool.insert(pool.end(), t.begin(), t.begin() + 2 * std::max(1, n - 1));
-    }
+    std::map<std::pair<int, int>, int> tw_off;  // (length, first radix of a two-stage pass or 0) -> offset
     hgrid.assign(G, BatchGrid{});
     for (int i = 0; i < G; ++i) {
         const int g = pgrid[i];
@@ -140,13 +130,23 @@ croft_status build_batch_tables(const std::vector<int>& dims, const std::vector<
             D.n[p] = n;
             D.M[p] = (axis == 2) ? 1 : (axis == 1 ? (long long)nz : (long long)ny * nz);
             D.ncols[p] = N / n;
-            D.tw_off[p] = off[n];
+            D.tw_off[p] = 0;
             D.dep[p] = -1;
+            if (n > CROFT_BATCH_MAX_N) return CROFT_ERR_UNSUPPORTED_SIZE;
             if (n == 1) {
                 D.W[p] = 1;
                 D.ntiles[p] = 0;
                 continue;
             }
+            const int r1 = croft_two_batch(n, D.M[p] == 1).r1;
+            const auto at = tw_off.emplace(std::make_pair(n, r1), (int)(pool.size() / 2));
+            if (at.second) {
+                std::vector<float> t(2 * (size_t)n + 2, 0.f);
+                if (r1) host_build_two_twiddles(n, r1, t.data());
+                else if (host_build_twiddles(n, t.data()) != n - 1) return CROFT_ERR_UNSUPPORTED_SIZE;
+                pool.insert(pool.end(), t.begin(), t.begin() + 2 * n);
+            }
+            D.tw_off[p] = at.first->second;
             const int T = croft_threads_per_pencil(n);
             D.W[p] = (D.M[p] == 1) ? CROFT_BATCH_THREADS / T : batch_col_width(n);
             D.ntiles[p] = (int)((D.ncols[p] + D.W[p] - 1) / D.W[p]);
@@ -405,7 +405,7 @@ static croft_status configure(BatchState* b, int mode) {
     }
     for (int g : b->sgrid) {
         croft_plan sp = nullptr;
-        // (a pass per axis, like the grouped launches: the same bits whichever mode is chosen)
+        // (a pass per axis, like the batch's schedules)
         croft_status st = croft_plan_create_schedule(&sp, b->dims[3 * g], b->dims[3 * g + 1], b->dims[3 * g + 2], CROFT_C2C_F32,
                                                      CROFT_SCHEDULE_THREE_PASS);
         if (st != CROFT_OK) return st;

@@ -112,7 +112,9 @@ int batch_smem_bytes() {
         const int T = croft_threads_per_pencil(N);                                                 \
         const int Wr = CROFT_BATCH_THREADS / T;                                                    \
         const int Wc = batch_col_width(N);                                                         \
-        int a = Wr * croft_row_ld_staged(N), b = N * Wc;                                           \
+        int ld = croft_row_ld_staged(N);                                                           \
+        if (croft_two_row(N).r1) ld = croft_two_batch_ld(N);                                       \
+        int a = Wr * ld, b = N * Wc;                                                               \
         int m = (a > b ? a : b) + tw;                                                              \
         if (m > best) best = m;                                                                    \
     }

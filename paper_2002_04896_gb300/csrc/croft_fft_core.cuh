@@ -63,17 +63,20 @@ struct GlobalInUnitT {  // unit stride (contiguous pencil)
 };
 // As GlobalIn, but read through L2 only (ld.global.cg): for data another CTA
 // wrote earlier in the same launch (the batched persistent kernel).
-struct GlobalInCG {
-    using value_type = float2;
+template <class C>
+struct GlobalInCGT {
+    using value_type = C;
     const float2* p;
     long long stride;
     float isign;
-    __device__ __forceinline__ float2 load(int a) const {
-        float2 t = __ldcg(p + (long long)a * stride);
-        t.y *= isign;
+    __device__ __forceinline__ C load(int a) const {
+        const float2 r = __ldcg(p + (long long)a * stride);
+        C t = mkc<C>(r.x, r.y);
+        conj_if(t, isign);
         return t;
     }
 };
+using GlobalInCG = GlobalInCGT<float2>;
 template <class C>
 struct GlobalOutT {
     using value_type = C;

@@ -62,7 +62,7 @@ __device__ __forceinline__ long long group_col_base(const GroupSeg& S, long long
 // The two-stage passes (croft_two_stage_kernel.cuh) of the lengths that have them: the same tiles
 // and arithmetic as a single grid's passes.
 template <int LAYOUT, int N>
-constexpr CroftTwo group_two() { return LAYOUT == LAYOUT_ROW ? croft_two_row(N) : croft_two_col(N, false); }
+constexpr CroftTwo group_two() { return croft_two_batch(N, LAYOUT == LAYOUT_ROW); }
 
 template <int LAYOUT, int N>
 __global__ void __launch_bounds__(group_two<LAYOUT, N>().w* group_two<LAYOUT, N>().t, group_two<LAYOUT, N>().minb)

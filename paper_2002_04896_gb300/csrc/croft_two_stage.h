@@ -184,6 +184,18 @@ CROFT_HD constexpr CroftTwo croft_two_row(int n) {
     }
 }
 
+// The entry of a batch's pass: its grids' strides are short.
+CROFT_HD constexpr CroftTwo croft_two_batch(int n, bool row) { return row ? croft_two_row(n) : croft_two_col(n, false); }
+// Row pencil's length in the exchange buffer of the persistent batched kernel, whose pencils take 4 or 8 threads: the
+// smallest distance at which the 16 threads of a half warp, on neighbouring pencils, meet no bank twice (one launch for 96 grids
+// of 64^3, distances of the row passes / these: 490 / 480 us).
+CROFT_HD constexpr int croft_two_batch_ld(int n) {
+    const int r1 = croft_two_row(n).r1, step = croft_threads_per_pencil(n) == 4 ? 8 : 16;
+    int ld = n / r1 * (r1 + (r1 % 2 == 0));
+    while (ld % step != step / 2) ++ld;
+    return ld;
+}
+
 // The fused convolution pass (croft_two_conv_kernel.cuh), x axis of n x 512 x 512; GB/s of its 20 bytes a
 // point (grid in and out, G in) of the three-stage kernel it replaced -> of this one.  Chosen for the long strides
 // of an x axis, the usual last axis; a 2D grid's y axis takes the same tiles.

@@ -102,6 +102,12 @@ struct TwoExCol {
     C* s;  // tile + c
     __device__ __forceinline__ C* at(int b, int j) const { return s + (b * R1 + j) * W; }
 };
+template <int R1, class C>
+struct TwoExColW {  // (width known at run time)
+    C* s;
+    int W;
+    __device__ __forceinline__ C* at(int b, int j) const { return s + (b * R1 + j) * W; }
+};
 // Rows: element b*R1 + j of a pencil at b*(R1 + D) + j.  An odd distance R1 + D between the
 // runs that neighbouring butterflies write keeps the writes free of bank conflicts.
 template <int R1, class C>

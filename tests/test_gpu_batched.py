@@ -109,6 +109,28 @@ def test_pme_batch_96_grouped_matches_single_grid_plans_bitwise(croft_lib, pme_b
         assert oracle.rel_l2(a[g].cpu().numpy(), oracle.forward(x)) <= tol(x.shape)
 
 
+BATCH_LENGTHS = [n for n in range(2, 129) if not [p for p in range(7, n + 1) if n % p == 0 and all(p % q for q in range(2, p))]]
+
+
+def test_every_mode_has_the_same_bits(croft_lib):
+    """Which schedule an AUTO plan times as the fastest does not change its results: every length as the z, y and x axis,
+    ragged tiles, both directions."""
+    dims = [d for n in BATCH_LENGTHS for d in ((5, 3, n), (2, n, 27), (n, 3, 25))] + [(64, 1, 1), (1, 60, 1), (108, 120, 125)]
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    ins = [torch.randn(d, dtype=torch.complex64, device="cuda", generator=gen) for d in dims]
+    ref = None
+    for mode in (croft_lib.CROFT_BATCH_GROUPED, croft_lib.CROFT_BATCH_PER_GRID, croft_lib.CROFT_BATCH_ONE_LAUNCH,
+                 croft_lib.CROFT_BATCH_PER_PASS):
+        with croft_lib.BatchPlan(dims, mode=mode) as p:
+            f, b = p.forward(ins), p.backward(ins)
+            torch.cuda.synchronize()
+            assert croft_lib.croft_plan_last_device_status(p.handle) == croft_lib.CROFT_OK
+        if ref is None:
+            ref = f, b
+        for d, t, u in zip(dims + dims, f + b, ref[0] + ref[1]):
+            assert torch.equal(torch.view_as_real(t), torch.view_as_real(u)), (mode, d)
+
+
 @pytest.mark.parametrize("count", [32, 33, 70])
 def test_grouped_batch_of_many_grids_of_one_length(croft_lib, count):
     """A launch holds 32 grids of one length: full, one over, and three launches per pass (y and z axes of 36 points)."""
