@@ -19,6 +19,9 @@
 // hides behind the forward stages.  The backward transform is conj(F(conj(.))):
 // the last forward stage stores conj(G * Y) into the tile, the forward stages
 // run again on it, and the final store conjugates.
+//
+// Complex64 axes of 36..1024 points run croft_two_conv_kernel.cuh instead (but 972 and 1000); this kernel serves the other
+// lengths and complex128.
 #pragma once
 #include <type_traits>
 
@@ -50,13 +53,11 @@ __device__ __forceinline__ void conv_cp_async(R* dst_smem, const R* src) {
 }
 
 // Launch shape: W = croft_conv_width(N) columns of T threads (a compile-time
-// constant, so every shared-memory index folds into constants).  For complex64
-// power-of-two lengths with 16-thread pencils (W = 16, 256-thread CTAs), asking
-// for four CTAs per SM keeps the kernel at 64 registers (72 at N = 256
-// otherwise: three CTAs per SM).  Complex64 pencils of 32 threads make 512-thread
-// CTAs whose tiles (data + G, ~100 KB at N = 512) allow two per SM, so they are
-// bound to two (64 registers).  Other lengths keep the 128-register bound:
-// radix-3/5 stages and complex128 spill at 64.
+// constant, so every shared-memory index folds into constants).  Complex64
+// power-of-two lengths in 256-thread CTAs ask for four CTAs per SM, which keeps the
+// kernel at 64 registers (at 256 points, before these had two stages, 72 otherwise:
+// three CTAs per SM).  Other lengths keep the 128-register bound: radix-3/5 stages and
+// complex128 spill at 64.
 template <int N, class C>
 struct ConvShape {
     static constexpr int T = croft_threads_per_pencil(N);
@@ -65,7 +66,7 @@ struct ConvShape {
     static constexpr bool TIGHT = sizeof(C) == 8 && THREADS == 256 && T <= 16 && (N & (N - 1)) == 0;
     // 0: no minimum in the launch bound (an explicit minimum of one or two lets ptxas
     // take far more registers than it does without one)
-    static constexpr int MIN_BLOCKS = TIGHT ? 4 : ((sizeof(C) == 8 && T == 32) ? 2 : 0);
+    static constexpr int MIN_BLOCKS = TIGHT ? 4 : 0;
 };
 
 // The last forward stage, the multiply by G and the first backward stage, in registers.

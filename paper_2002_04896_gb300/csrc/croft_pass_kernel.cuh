@@ -78,9 +78,10 @@ __device__ __forceinline__ void pass_body(const C* in, C* out, const PassArgs& A
     }
 }
 
-// BACK: the kernel follows A.backwards (col_tile).  The kernels without a minimum of CTAs per SM - lengths of short
-// passes inside the L2 among them - do not: choosing the tile ahead of every address costs a 128^3 transform
-// 0.9 of its 19 us.
+// BACK: the kernel follows A.backwards (col_tile).  The bounded kernels do.  The others - in default plans complex128 and
+// the lengths without a two-stage kernel: up to 32, 972, 1000 and beyond 1024 points - do not: where it was measured, at 128
+// points before that length had a two-stage kernel, choosing the tile ahead of every address cost a 128^3 transform 0.9
+// of its 19 us.  Their own lengths have not been measured with it.
 //
 // The pass kernel.  (Its launch bound names no minimum of CTAs per SM: with an
 // explicit minimum of one, ptxas allocates far more registers - 83 instead of 52

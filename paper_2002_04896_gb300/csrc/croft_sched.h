@@ -149,6 +149,11 @@ CROFT_HD constexpr int croft_threads_per_pencil(int n) {
     return p;
 }
 
+// The rules from here on choose among the general kernels (croft_pass_kernel.cuh and its
+// kin).  Default complex64 plans run two-stage kernels at 36..1024 points (croft_two_stage.h)
+// and follow these rules at the other lengths only; at 36..1024 points they act where the
+// two-stage kernels are off (CROFT_TWO_STAGE=0), and their kernels are a tuned plan's candidates.
+//
 // The schedule of a pass over a length-n axis (layout 0 = ROW, 1 = COL; es = complex
 // element size): the column passes of complex64 32-thread pencils (lengths 270..512,
 // bounded to 40 registers) take the near-equal power-of-two split - at 480 the
@@ -184,7 +189,8 @@ CROFT_HD constexpr CroftSched croft_pass_sched_v(int n, int layout, int es, int 
 // (16·5·4 against 8·8·5, 16-column tiles: y of 512 x 320 x 512 231 / 260 us, x of 320 x 512 x
 // 512 240 / 287); the 512-point short-stride pass, variant 2 (16·8·4; 8-column tiles: 512^3 y
 // 387 us against 391 for 16·16·2 and 399 for 8·8·8).  Twiddle tables follow the pass's
-// variant; a fused convolution on such an axis gets a table of its own.
+// variant; the fused convolution of these lengths has a split and a table of its own
+// (croft_two_conv).
 CROFT_HD constexpr int croft_col_sv_default(int n, int es, long long stride_bytes) {
     return (es == 8 && n == 512 && stride_bytes <= 16 * 1024) ? 2 : ((es == 8 && n == 320) ? 1 : 0);
 }
