@@ -33,7 +33,7 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
 }
 
 // complex64 whose sums and differences take one instruction for both parts (add and fma .f32x2 of sm_100 and later; the
-// same roundings as float2's).  Kernels that are bound by instruction issue or by the length of their
+// same roundings as float2's, whose products the butterflies below fuse with their sums explicitly).  Kernels that are bound by instruction issue or by the length of their
 // butterflies gain a few per cent, kernels short of registers lose to the pairing: each two-stage kernel
 // has the measured choice in its table (croft_two_stage.h).
 struct __align__(8) packed2 {
@@ -197,10 +197,11 @@ template <class C> struct Dft<3, C> {
         C t = cadd(v[1], v[2]);
         C d = csub(v[1], v[2]);
         C m = mkc<C>(fma((T)-0.5, t.x, v[0].x), fma((T)-0.5, t.y, v[0].y));
-        C r = mkc<C>(r3 * d.y, -r3 * d.x);  // -i * (sqrt3/2) * d
         v[0] = cadd(v[0], t);
-        v[1] = cadd(m, r);
-        v[2] = csub(m, r);
+        // m -+ i (sqrt3/2) d as multiply-adds, one rounding each (paired sums of the rounded products would
+        // take as many instructions and round twice)
+        v[1] = mkc<C>(fma(r3, d.y, m.x), fma(-r3, d.x, m.y));
+        v[2] = mkc<C>(fma(-r3, d.y, m.x), fma(r3, d.x, m.y));
     }
 };
 
