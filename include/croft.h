@@ -385,8 +385,8 @@ croft_status croft_exec_host_pipeline(croft_plan plan, int count, const void* co
  * its three grid buffers). */
 size_t croft_plan_workspace_bytes(croft_plan plan);
 
-/* Number of kernel launches one exec of this plan issues (with timing enabled, croft_plan_set_timing,
- * AUTO plans take one launch per axis). */
+/* Number of kernel launches one forward or backward exec of this plan issues (with timing enabled,
+ * croft_plan_set_timing, AUTO plans take one launch per axis). */
 int croft_plan_num_launches(croft_plan plan);
 
 /*

@@ -110,6 +110,7 @@ struct PlanePass {
     plane_pass_fn fn;    // NULL: none
     PlanePassArgs args;  // (in, out and isign filled per exec)
     int grid, block, smem;
+    bool transforms, convolutions;  // which of the two run it (croft_plane_pass_rule)
 };
 
 // The two-stage kernel that runs an axis pass in place of its three-stage one (croft_two_stage.h).

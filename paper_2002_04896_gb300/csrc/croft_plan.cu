@@ -386,9 +386,11 @@ static croft_status add_slab_passes(croft_plan p, int planes) {
     return CROFT_OK;
 }
 
-// Whether an exec runs the z and y axes as one pass over the planes: not while it times every axis
-// (croft_plan_set_timing), which takes a launch per axis.
-static bool zy_runs(const croft_plan p) { return p->zy.fn && !p->timing; }
+// Whether a transform or a convolution runs the z and y axes as one pass over the planes: not while it times every
+// axis (croft_plan_set_timing), which takes a launch per axis.
+static bool zy_runs(const croft_plan p, bool convolution) {
+    return p->zy.fn && !p->timing && (convolution ? p->zy.convolutions : p->zy.transforms);
+}
 
 // The z+y pass over whole planes (croft_plane_pass_kernel.cuh), beside the z and y passes that
 // croft_exec_axes and per-axis timing run: AUTO plans of complex64 grids whose planes it takes.
@@ -397,9 +399,11 @@ static croft_status plan_zy(croft_plan p) {
     const int nx = p->dims[0], ny = p->dims[1], nz = p->dims[2];
     const char* pe = getenv("CROFT_PLANE_PASS");
     if ((pe && pe[0] == '0') || p->passes.size() < 2 || p->pass_axis[0] != 2 || p->pass_axis[1] != 1) return CROFT_OK;
-    if (!croft_plane_pass_rule(nx, ny, nz, device_sms())) return CROFT_OK;
     PlanePass z;
     memset(&z, 0, sizeof(z));
+    z.transforms = croft_plane_pass_rule(nx, ny, nz, device_sms(), false);
+    z.convolutions = nx > 1 && croft_plane_pass_rule(nx, ny, nz, device_sms(), true);  // (one plane: the fused pass takes y)
+    if (!z.transforms && !z.convolutions) return CROFT_OK;
     z.smem = croft_plane_smem(ny, nz);
     if (z.smem > g_max_smem) return CROFT_OK;
     if (plane_pass_prepare(ny, z.smem) != cudaSuccess) {
@@ -931,7 +935,7 @@ static croft_status create_tuned(croft_plan* out, int nx, int ny, int nz, croft_
                                       CROFT_SCHEDULE_AUTO};
     static const char* sn[4] = {"three_pass", "slab_l2", "plane_fused", "plane_pass"};
     double best = 1e30;
-    for (int k = 0; k < (croft_plane_pass_rule(nx, ny, nz, device_sms()) ? 4 : 3); ++k) {
+    for (int k = 0; k < (croft_plane_pass_rule(nx, ny, nz, device_sms(), false) ? 4 : 3); ++k) {
         croft_plan p = nullptr;
         const croft_status st = create_impl(&p, nx, ny, nz, dtype, scheds[k], (k == 0 || k == 3) ? &ch : nullptr);
         if (st != CROFT_OK) {
@@ -1008,7 +1012,8 @@ int croft_plan_describe(croft_plan plan, char* buf, int cap) {
         }
     }
     if (plan->zy.fn) {
-        snprintf(tmp, sizeof(tmp), " | z+y in one pass over the planes: %dx%d, %dx%d block=%d grid=%d smem=%d",
+        snprintf(tmp, sizeof(tmp), " | %sz+y in one pass over the planes: %dx%d, %dx%d block=%d grid=%d smem=%d",
+                 plan->zy.transforms ? (plan->zy.convolutions ? "" : "transforms: ") : "convolutions: ",
                  croft_plane_r1z(plan->dims[2]), plan->dims[2] / croft_plane_r1z(plan->dims[2]), croft_plane_r1y(plan->dims[1]),
                  plan->dims[1] / croft_plane_r1y(plan->dims[1]), plan->zy.block, plan->zy.grid, plan->zy.smem);
         s += tmp;
@@ -1048,7 +1053,7 @@ size_t croft_plan_workspace_bytes(croft_plan plan) {
 int croft_plan_num_launches(croft_plan plan) {
     if (!plan) return -1;
     if (plan->batch) return batch_num_launches(plan);
-    return (int)plan->passes.size() - (zy_runs(plan) ? 1 : 0);
+    return (int)plan->passes.size() - (zy_runs(plan, false) ? 1 : 0);
 }
 
 croft_status croft_plan_set_timing(croft_plan plan, int enable) {
@@ -1101,8 +1106,8 @@ croft_status croft_plan_last_device_status(croft_plan plan) {
 // device for that pass's results.  The first launch of an exec is ordered after
 // the caller's earlier work in the ordinary way.
 static croft_status run_passes(croft_plan plan, size_t i0, size_t i1, const void* in, void* out, cudaStream_t s,
-                               float isign, bool force_out, int* evi, bool& started) {
-    if (i0 == 0 && i1 >= 2 && zy_runs(plan)) {  // z and y as one pass
+                               float isign, bool convolution, bool force_out, int* evi, bool& started) {
+    if (i0 == 0 && i1 >= 2 && zy_runs(plan, convolution)) {  // z and y as one pass
         const bool pdl = plan->pdl && started;
         started = true;
         if (launch_plane_pass(plan->zy, (const float2*)(force_out ? out : in), (float2*)out, isign, s, pdl) != cudaSuccess) {
@@ -1164,7 +1169,7 @@ static croft_status exec_dir(croft_plan plan, const void* in, void* out, void* s
         evi = 1;
     }
     bool started = false;
-    croft_status st = run_passes(plan, 0, plan->passes.size(), in, out, s, isign, false, tm ? &evi : nullptr, started);
+    croft_status st = run_passes(plan, 0, plan->passes.size(), in, out, s, isign, false, false, tm ? &evi : nullptr, started);
     if (st != CROFT_OK) return st;
     plan->ev_count = tm ? evi : 0;
     plan->ran = true;
@@ -1197,7 +1202,7 @@ croft_status croft_exec_convolve(croft_plan plan, const void* in, void* out, con
     if (plan->conv_fused) {
         // forward passes but the last, the fused last-axis pass, backward passes of the other axes
         const size_t last = plan->passes.size() - 1;
-        st = run_passes(plan, 0, last, in, out, s, 1.0f, false, pe, started);
+        st = run_passes(plan, 0, last, in, out, s, 1.0f, true, false, pe, started);
         if (st != CROFT_OK) return st;
         const PassLaunch& L = plan->conv;
         if (launch_conv(L, L.src_in ? in : out, out, g, s, plan->pdl && started) != cudaSuccess) {
@@ -1206,11 +1211,11 @@ croft_status croft_exec_convolve(croft_plan plan, const void* in, void* out, con
         }
         started = true;
         if (tm && cudaEventRecord(plan->ev[evi++], s) != cudaSuccess) { cudaGetLastError(); return CROFT_ERR_CUDA; }
-        st = run_passes(plan, 0, last, in, out, s, -1.0f, true, pe, started);
+        st = run_passes(plan, 0, last, in, out, s, -1.0f, true, true, pe, started);
         if (st != CROFT_OK) return st;
     } else {
         // F, multiply, B (a one-point grid has no passes: the multiply reads `in`)
-        st = run_passes(plan, 0, plan->passes.size(), in, out, s, 1.0f, false, pe, started);
+        st = run_passes(plan, 0, plan->passes.size(), in, out, s, 1.0f, true, false, pe, started);
         if (st != CROFT_OK) return st;
         // (after a tensor-core pass, which does not wait on the device, the multiply is ordered normally)
         const bool pdl = plan->pdl && started && pass_supports_pdl(plan->passes.back());
@@ -1220,7 +1225,7 @@ croft_status croft_exec_convolve(croft_plan plan, const void* in, void* out, con
         }
         started = true;
         if (tm && cudaEventRecord(plan->ev[evi++], s) != cudaSuccess) { cudaGetLastError(); return CROFT_ERR_CUDA; }
-        st = run_passes(plan, 0, plan->passes.size(), in, out, s, -1.0f, true, pe, started);
+        st = run_passes(plan, 0, plan->passes.size(), in, out, s, -1.0f, true, true, pe, started);
         if (st != CROFT_OK) return st;
     }
     plan->ev_count = tm ? evi : 0;

@@ -22,7 +22,7 @@
 // HBM are contiguous and a warp shares its twiddles), each a walk of odd stride over the banks.
 //
 // The kernel is specialised on ny; the z stages are functions of their own, one per nz, called once
-// per plane (20 kernels and 13 such functions instead of a kernel for every pair of lengths).
+// per plane (20 kernels and 16 such functions instead of a kernel for every pair of lengths).
 #pragma once
 #include "croft_butterflies.cuh"
 #include "croft_fft_core.cuh"
@@ -71,7 +71,8 @@ __device__ __noinline__ void plane_z(const float2* in, const float2* tw, int ny,
 #define CROFT_PLANE_Y_SIZES(X)                                                                                   \
     X(32) X(36) X(40) X(45) X(48) X(50) X(54) X(60) X(64) X(72) X(75) X(80) X(81) X(90) X(96) X(100) X(108)      \
     X(120) X(125) X(128)
-#define CROFT_PLANE_Z_SIZES(X) X(32) X(36) X(40) X(45) X(48) X(50) X(54) X(60) X(64) X(72) X(75) X(81) X(125)
+#define CROFT_PLANE_Z_SIZES(X)                                                                                   \
+    X(32) X(36) X(40) X(45) X(48) X(50) X(54) X(60) X(64) X(72) X(75) X(80) X(81) X(90) X(96) X(125)
 
 template <int NY>
 __global__ void __launch_bounds__(1024) croft_plane_pass_kernel(const __grid_constant__ PlanePassArgs A) {

@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 Y_LENGTHS = [32, 36, 40, 45, 48, 50, 54, 60, 64, 72, 75, 80, 81, 90, 96, 100, 108, 120, 125, 128]
-Z_LENGTHS = [32, 36, 40, 45, 48, 50, 54, 60, 64, 72, 75, 81, 125]
+Z_LENGTHS = [32, 36, 40, 45, 48, 50, 54, 60, 64, 72, 75, 80, 81, 90, 96, 125]
 
 
 def _noise(shape, seed):
@@ -20,12 +20,34 @@ def _noise(shape, seed):
     return (rng.uniform(-1, 1, shape) + 1j * rng.uniform(-1, 1, shape)).astype(np.complex64)
 
 
+def _takes(croft, shape):
+    """Whether an AUTO plan's transforms and its convolutions run z and y as one pass."""
+    with croft.Plan(*shape) as p:
+        part = [s for s in p.describe().split(" | ") if "z+y in one pass" in s]
+    return bool(part) and not part[0].startswith("convolutions: "), bool(part) and not part[0].startswith("transforms: ")
+
+
+def _check_convolution(croft, shape):
+    assert _takes(croft, shape)[1], shape
+    x = _noise(shape, sum(shape))
+    g = np.random.default_rng(6).uniform(0.1, 1, shape).astype(np.float32)
+    d, dg = torch.from_numpy(x).cuda(), torch.from_numpy(g).cuda()
+    with croft.Plan(*shape) as p, croft.Plan(*shape, schedule=croft.CROFT_SCHEDULE_THREE_PASS) as q:
+        assert "fwd*G*bwd fused" in p.describe()
+        y, z = p.convolve(d, dg), q.convolve(d, dg)
+        p.convolve(d, dg, d)  # in place
+        torch.cuda.synchronize()
+    assert torch.equal(torch.view_as_real(y), torch.view_as_real(z)), shape
+    assert torch.equal(torch.view_as_real(y), torch.view_as_real(d)), shape
+    assert oracle.rel_l2(y.cpu().numpy(), oracle.convolve(x, g)) <= 4e-6 * math.log2(x.size), shape
+
+
 def _check(croft, shape):
     x = _noise(shape, sum(shape))
     tol = 2e-6 * math.log2(x.size)
     d = torch.from_numpy(x).cuda()
+    assert _takes(croft, shape)[0], shape
     with croft.Plan(*shape) as p:
-        assert "z+y in one pass" in p.describe(), p.describe()
         assert croft.croft_plan_num_launches(p.handle) == (2 if shape[0] > 1 else 1)
         out = torch.full_like(d, complex(float("nan"), 0))
         p.forward(d, out)
@@ -60,31 +82,34 @@ def test_every_length_as_y(croft_lib, n):
 
 @pytest.mark.parametrize("n", Z_LENGTHS)
 def test_every_length_as_z(croft_lib, n):
-    _check(croft_lib, (2, 32, n) if n <= 72 else (400, 36, n))
+    if n <= 81:
+        _check(croft_lib, (2, 32, n))
+    elif n != 90:
+        _check(croft_lib, (320, 36, n))
     if n <= 36:
         _check(croft_lib, (1, n, n))
+    _check_convolution(croft_lib, (24 if n != 125 else 80, 32, n))
 
 
 # one plane an SM and a rest; 256- and 128-thread CTAs; the largest planes the rule takes
-@pytest.mark.parametrize("shape", [(150, 100, 45), (256, 80, 60), (300, 128, 36), (480, 96, 50), (480, 36, 125), (625, 36, 45),
+@pytest.mark.parametrize("shape", [(150, 80, 54), (256, 80, 60), (300, 128, 36), (480, 96, 50), (480, 36, 125), (625, 36, 45),
                                    (480, 128, 32), (100, 36, 64)])
 def test_many_planes(croft_lib, shape):
     _check(croft_lib, shape)
 
 
-def test_convolution_and_rule(croft_lib):
-    shape = (20, 48, 45)
-    x = _noise(shape, 5)
-    g = np.random.default_rng(6).uniform(0.1, 1, shape).astype(np.float32)
-    with croft_lib.Plan(*shape) as p:
-        assert "z+y in one pass" in p.describe() and "fwd*G*bwd fused" in p.describe()
-        y = p.convolve(torch.from_numpy(x).cuda(), torch.from_numpy(g).cuda())
-        torch.cuda.synchronize()
-    assert oracle.rel_l2(y.cpu().numpy(), oracle.convolve(x, g)) <= 4e-6 * math.log2(x.size)
-    for shape, takes in (((48, 48, 48), True), ((60, 60, 60), False), ((16, 64, 64), False), ((120, 48, 48), False),
-                         ((120, 100, 32), True), ((128, 60, 54), True), ((300, 48, 36), True), ((300, 64, 64), False),
-                         ((300, 108, 108), False), ((8, 30, 32), False), ((8, 32, 256), False)):
-        with croft_lib.Plan(*shape) as p:
-            assert ("z+y in one pass" in p.describe()) == takes, shape
+@pytest.mark.parametrize("shape", [(108, 54, 54), (160, 90, 45), (240, 45, 90), (320, 64, 75), (400, 40, 48), (640, 50, 60)])
+def test_convolutions_of_many_planes(croft_lib, shape):
+    _check_convolution(croft_lib, shape)
+
+
+def test_rule(croft_lib):
+    """(transforms, convolutions) of AUTO plans; other schedules run axis by axis."""
+    for shape, takes in (((48, 48, 48), (True, True)), ((60, 60, 60), (False, False)), ((16, 64, 64), (False, False)),
+                         ((80, 64, 64), (False, True)), ((120, 48, 48), (False, True)), ((120, 100, 32), (True, True)),
+                         ((128, 60, 54), (True, False)), ((300, 48, 36), (True, True)), ((300, 64, 64), (False, False)),
+                         ((300, 108, 108), (False, False)), ((8, 30, 32), (False, False)), ((8, 32, 256), (False, False)),
+                         ((1, 36, 36), (True, False))):
+        assert _takes(croft_lib, shape) == takes, shape
         with croft_lib.Plan(*shape, schedule=croft_lib.CROFT_SCHEDULE_THREE_PASS) as p:
             assert "z+y in one pass" not in p.describe(), shape

@@ -66,12 +66,13 @@ PLANE_PROGRAM = r"""
 int main() {
     const int sms[2] = {152, 148};
     for (int s : sms)
-        for (int nx = 1; nx <= 1200; ++nx)
-            for (int ny = 1; ny <= 140; ++ny)
-                for (int nz = 1; nz <= 140; ++nz)
-                    if (croft_plane_pass_rule(nx, ny, nz, s))
-                        std::printf("%d %d %d %d %d %d %d %d\n", s, nx, ny, nz, croft_plane_r1y(ny), croft_plane_r1z(nz),
-                                    croft_plane_smem(ny, nz), croft_plane_threads(nx, ny, nz, s));
+        for (int conv = 0; conv < 2; ++conv)
+            for (int nx = 1; nx <= 1200; ++nx)
+                for (int ny = 1; ny <= 140; ++ny)
+                    for (int nz = 1; nz <= 140; ++nz)
+                        if (croft_plane_pass_rule(nx, ny, nz, s, conv != 0))
+                            std::printf("%d %d %d %d %d %d %d %d %d\n", s, conv, nx, ny, nz, croft_plane_r1y(ny), croft_plane_r1z(nz),
+                                        croft_plane_smem(ny, nz), croft_plane_threads(nx, ny, nz, s));
     return 0;
 }
 """
@@ -85,19 +86,22 @@ def test_plane_rule_edges(tmp_path):
     subprocess.run([cxx, "-std=c++17", "-I", CSRC, str(tmp_path / "p.cpp"), "-o", str(tmp_path / "p")], check=True)
     out = subprocess.run([str(tmp_path / "p")], check=True, capture_output=True, text=True).stdout
     rows = [tuple(map(int, line.split())) for line in out.splitlines()]
-    took = {r[:4] for r in rows}
-    for _, nx, ny, nz, r1y, r1z, smem, threads in rows:
+    took = {r[:5] for r in rows}
+    for _, _, nx, ny, nz, r1y, r1z, smem, threads in rows:
         assert r1y in RADICES and r1z in RADICES and ny % r1y == 0 and nz % r1z == 0 and max(ny // r1y, nz // r1z) <= 25
         assert smem <= 99 * 1024 and threads in (128, 256, 512), (nx, ny, nz)
         assert ny * nz <= 4800 and nx * ny * nz <= 4 * 1024 * 1024
-    # the number of planes up to which small planes are taken (two SMs of three), rows of 32 points (five of six), and from which
-    # the longer planes are, follows the device
+    assert {r[4] for r in rows} == {32, 36, 40, 45, 48, 50, 54, 60, 64, 72, 75, 80, 81, 90, 96, 125}
+    # the number of planes up to which small planes are taken (two SMs of three) or rows of 32 points (five of six), and from
+    # which the longer planes are, follows the device
     for sms, few, rows32, many in ((152, 101, 126, 456), (148, 98, 123, 444)):
-        assert (sms, few, 48, 48) in took and (sms, few + 1, 48, 48) not in took and (sms, few, 50, 48) not in took
-        assert (sms, rows32, 128, 32) in took and (sms, rows32 + 1, 128, 32) not in took
-        assert (sms, many, 90, 50) in took and (sms, many - 1, 90, 50) not in took
-        assert (sms, 1, 48, 32) in took and (sms, 1, 48, 36) not in took
-        assert not any(r[0] == sms and r[3] in (80, 90, 96, 100, 108, 120, 128) for r in rows)
+        t, c = (sms, 0), (sms, 1)  # transforms, convolutions
+        assert t + (few, 48, 48) in took and t + (few + 1, 48, 48) not in took and t + (few, 50, 48) not in took
+        assert t + (few, 64, 54) in took and t + (few, 72, 54) not in took and t + (18, 54, 54) not in took and t + (few, 36, 72) not in took
+        assert c + (few, 64, 64) in took and c + (few + 1, 64, 64) not in took and c + (few + 1, 48, 64) in took
+        assert t + (rows32, 128, 32) in took and t + (rows32 + 1, 128, 32) not in took and c + (rows32 + 1, 128, 32) in took
+        assert t + (many, 90, 50) in took and t + (many - 1, 90, 50) not in took and c + (many - 1, 90, 50) in took
+        assert t + (1, 36, 60) in took and t + (1, 48, 40) not in took and t + (1, 32, 48) in took
 
 
 def test_half_tiles_follow_the_sm_count(tmp_path):
