@@ -394,11 +394,12 @@ static bool zy_runs(const croft_plan p, bool convolution) {
 
 // The z+y pass over whole planes (croft_plane_pass_kernel.cuh), beside the z and y passes that
 // croft_exec_axes and per-axis timing run: AUTO plans of complex64 grids whose planes it takes.
-// CROFT_PLANE_PASS=0 switches it off (measurement).
+// CROFT_PLANE_PASS=0 switches it off (measurement), and so does CROFT_TWO_STAGE=0.
 static croft_status plan_zy(croft_plan p) {
     const int nx = p->dims[0], ny = p->dims[1], nz = p->dims[2];
     const char* pe = getenv("CROFT_PLANE_PASS");
     if ((pe && pe[0] == '0') || p->passes.size() < 2 || p->pass_axis[0] != 2 || p->pass_axis[1] != 1) return CROFT_OK;
+    if (!two_selected(p, 1) || !two_selected(p, 2)) return CROFT_OK;  // (its bits are those of the two-stage passes)
     PlanePass z;
     memset(&z, 0, sizeof(z));
     z.transforms = croft_plane_pass_rule(nx, ny, nz, device_sms(), false);
@@ -708,7 +709,7 @@ static croft_status create_impl(croft_plan* out, int nx, int ny, int nz, croft_d
         croft_status st = add_axis_pass(p, axes[i]);
         if (st != CROFT_OK) return fail(p, st);
     }
-    if (sched == CROFT_SCHEDULE_AUTO && !fused && !want_tc && dtype == CROFT_C2C_F32 && p->axis_kind[1] < 0 && p->axis_kind[2] < 0) {
+    if (sched == CROFT_SCHEDULE_AUTO && !fused && !want_tc && dtype == CROFT_C2C_F32) {
         const croft_status st = plan_zy(p);
         if (st != CROFT_OK) return fail(p, st);
     }

@@ -121,6 +121,8 @@ def test_switches_name_their_own_kernels_only(croft_lib, monkeypatch, switch, ke
     assert d.count("-> two-stage") == two, d
     assert ("-> two-stage" in x) == (kernel is None and two > 0), d
     assert kernel is None or kernel in x, d
+    with croft_lib.Plan(48, 48, 48) as p:  # the plane pass has the two-stage passes' bits, and goes with them
+        assert ("z+y in one pass" in p.describe()) == (two > 0), p.describe()
 
 
 def test_slab_plans_build_each_table_once(croft_lib, monkeypatch):
